@@ -28,26 +28,53 @@ struct PhysParams {
 
 // ---------------------------------------------------------------------------
 // Logarithmic mean L(a,b) = (a-b)/(ln a - ln b) and its inverse.
-// For a ~ b both use the series in u = ((a-b)/(a+b))^2:
-//   L = (a+b) / (2 F(u)),  F(u) = 1 + u/3 + u^2/5 + u^3/7 + ...
-// FP64: 4 terms below u = 1e-4 (truncation u^4/9 < 1.2e-17).
+// For a ~ b both use polynomials in u = ((a-b)/(a+b))^2:
+//   L = (a+b) / (2 F(u)),  F(u) = artanh(sqrt u) / sqrt u = 1 + u/3 + u^2/5 + ...
+//   and 1/F(u) = 1 - u/3 - 4u^2/45 - ...
+// FP64: degree 8 below u = 1/16 (least-maximum fits on [0, 1/16], computed with
+// 50 digits; error below 9e-18), inside it degree 3 below u = 2^-13 (error
+// below 2e-19); above 1/16 the ratio a/b exceeds 1.66 and log(a/b) is well
+// conditioned (at u = 1e-4 the quotient's rounding costs log(a/b) 1e-16 / 0.02).
 // FP32: 5 terms below u = 0.05 (truncation below u^5 / (11 (1 - u)) < 3e-8,
-// half an FP32 ulp of F ~ 1); above it the ratio a/b exceeds 1.57 and
-// log(a/b) is well conditioned.
+// half an FP32 ulp of F ~ 1); above it the ratio a/b exceeds 1.57.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double series_F(double u) {
-  return 1.0 + u * (1.0 / 3.0 + u * (1.0 / 5.0 + u * (1.0 / 7.0)));
+  return 1.0 + u * (0.33333333333331369 + u * (0.20000000000836662 + u * (0.14285714148744664 + u * (0.11111122319976208
+      + u * (0.090903954153249859 + u * (0.077060649643451390 + u * (0.064540716251361030 + u * 0.076102246025017837)))))));
+}
+__device__ __forceinline__ double series_invF(double u) {
+  return 1.0 + u * (-0.33333333333332982 + u * (-0.088888888890384454 + u * (-0.046560846315972715 + u * (-0.030194023571221005
+      + u * (-0.021795885119032539 + u * (-0.016812176252078610 + u * (-0.013121851935549912 + u * -0.014306111787604733)))))));
+}
+// u < 2^-13
+__device__ __forceinline__ double series_F_near(double u) {
+  return 1.0 + u * (0.33333333333338387 + u * (0.19999999793002216 + u * 0.14288427331899907));
+}
+__device__ __forceinline__ double series_invF_near(double u) {
+  return 1.0 + u * (-0.33333333333334706 + u * (-0.088888888326392527 + u * -0.046568219037031879));
 }
 __device__ __forceinline__ float series_F(float u) {
   return 1.0f + u * (1.0f / 3.0f + u * (1.0f / 5.0f + u * (1.0f / 7.0f + u * (1.0f / 9.0f))));
 }
+// 1/F(u) by its own series (five terms; the truncation is below 7e-9 relative
+// for u < 0.05), so that the series branch needs a single reciprocal
+__device__ __forceinline__ float series_invF(float u) {
+  return 1.0f + u * (-1.0f / 3.0f + u * (-4.0f / 45.0f + u * (-44.0f / 945.0f + u * (-428.0f / 14175.0f))));
+}
 template <typename R> struct LogMeanEps;
-template <> struct LogMeanEps<double> { static constexpr double v = 1e-4; };
+template <> struct LogMeanEps<double> { static constexpr double v = 0.0625; };
 template <> struct LogMeanEps<float> { static constexpr float v = 0.05f; };
 
-// FP64: IEEE division.  FP32: the MUFU reciprocal (rcp.approx, about 1 ulp),
-// no slow-path branch.
-__device__ __forceinline__ double fast_rcp(double x) { return 1.0 / x; }
+// FP64: the reciprocal unit's approximation r of 1/x (relative error about
+// 2^-20) and one third-order Householder iteration, r (1 + e + e^2) with
+// e = 1 - x r: three FP64 fused multiply-adds, error e^3 plus one rounding.
+// FP32: the MUFU reciprocal (rcp.approx, about 1 ulp), no slow-path branch.
+__device__ __forceinline__ double fast_rcp(double x) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
 __device__ __forceinline__ float fast_rcp(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -62,7 +89,7 @@ __device__ __forceinline__ R logmean(R a, R b) {
   R rs = fast_rcp(s);
   R f = d * rs;
   R u = f * f;
-  if (u < LogMeanEps<R>::v) return R(0.5) * s * fast_rcp(series_F(u));
+  if (u < LogMeanEps<R>::v) return R(0.5) * s * series_invF(u);
   return d * fast_rcp(plain_log(a * fast_rcp(b)));
 }
 
@@ -84,29 +111,9 @@ __device__ __noinline__ void logmean_pair_general(R a1, R b1, R a2, R b2, R& L1,
   iL2 = inv_logmean(a2, b2);
 }
 
-// L(a1,b1) and 1/L(a2,b2) together: one branch decides for both whether the
-// series applies (the common case on resolved data), otherwise each takes its
-// own branch above.
-template <typename R>
-__device__ __forceinline__ void logmean_pair(R a1, R b1, R a2, R b2, R& L1, R& iL2) {
-  R s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
-  R rs1 = fast_rcp(s1), rs2 = fast_rcp(s2);
-  R f1 = d1 * rs1, f2 = d2 * rs2;
-  R u1 = f1 * f1, u2 = f2 * f2;
-  if (fmax(u1, u2) < LogMeanEps<R>::v) {
-    L1 = R(0.5) * s1 * fast_rcp(series_F(u1));
-    iL2 = R(2) * series_F(u2) * rs2;
-  } else {
-    logmean_pair_general(a1, b1, a2, b2, L1, iL2);
-  }
-}
-
-// FP32: 1/F(u) = sqrt(u)/artanh(sqrt(u)) by its own series (five terms; the
-// truncation is below 7e-9 relative for u < 0.05), so that the series branch
-// needs a single reciprocal: 1/(s1 s2) gives both 1/s1 and 1/s2.
-__device__ __forceinline__ float series_invF(float u) {
-  return 1.0f + u * (-1.0f / 3.0f + u * (-4.0f / 45.0f + u * (-44.0f / 945.0f + u * (-428.0f / 14175.0f))));
-}
+// L(a1,b1) and 1/L(a2,b2) together: one reciprocal, 1/(s1 s2), gives both 1/s1
+// and 1/s2, and one branch decides for both which form applies (the series on
+// resolved data; otherwise each takes its own branch above).
 __device__ __forceinline__ void logmean_pair(float a1, float b1, float a2, float b2, float& L1, float& iL2) {
   const float s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
   const float r = fast_rcp(s1 * s2);
@@ -121,21 +128,38 @@ __device__ __forceinline__ void logmean_pair(float a1, float b1, float a2, float
   }
 }
 
-// FP64: the same single-reciprocal form (each FP64 division is a dozen
-// instructions on the narrow FP64 pipe): 1/F(u) by its own series, five terms
-// (truncation below 1e-21 for u < 1e-4), and 1/s1, 1/s2 from 1/(s1 s2).
-__device__ __forceinline__ double series_invF(double u) {
-  return 1.0 + u * (-1.0 / 3.0 + u * (-4.0 / 45.0 + u * (-44.0 / 945.0 + u * (-428.0 / 14175.0))));
+// the wide polynomials of both means, out of line (twenty instructions on the
+// FP64 pipe that most pairs of a resolved flow do not need)
+static __device__ __noinline__ void series_pair_wide(double u1, double u2, double& g1, double& f2) {
+  g1 = series_invF(u1);
+  f2 = series_F(u2);
 }
+
+// FP64: the branch compares the high words (u >= 0, and a NaN's is above every
+// bound), which keeps the comparisons off the narrow FP64 pipe that bounds
+// these kernels.  A flow resolved by its mesh mixes pairs below 2^-13 (two
+// thirds of them on the 256^2, N = 3 shear layer) with pairs up to 1e-2; sending
+// the latter to two logarithms (about 150 FP64 instructions with their
+// divisions) instead of the wide polynomials, as a single bound of 1e-4 did,
+// took 124 against 71 us per volume launch on the 64-element 1D wave and 2138
+// against 1846 us on the shear layer (with the three-FMA reciprocal).
 __device__ __forceinline__ void logmean_pair(double a1, double b1, double a2, double b2, double& L1, double& iL2) {
   const double s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
-  const double r = 1.0 / (s1 * s2);
+  const double r = fast_rcp(s1 * s2);
   const double rs1 = s2 * r, rs2 = s1 * r;
   const double f1 = d1 * rs1, f2 = d2 * rs2;
   const double u1 = f1 * f1, u2 = f2 * f2;
-  if (fmax(u1, u2) < LogMeanEps<double>::v) {
-    L1 = 0.5 * s1 * series_invF(u1);
-    iL2 = 2.0 * series_F(u2) * rs2;
+  const unsigned h = max((unsigned)__double2hiint(u1), (unsigned)__double2hiint(u2));
+  if (h < 0x3FB00000u) {   // 1/16
+    double g, f;
+    if (h < 0x3F200000u) {   // 2^-13
+      g = series_invF_near(u1);
+      f = series_F_near(u2);
+    } else {
+      series_pair_wide(u1, u2, g, f);
+    }
+    L1 = 0.5 * s1 * g;
+    iL2 = 2.0 * f * rs2;
   } else {
     logmean_pair_general(a1, b1, a2, b2, L1, iL2);
   }
@@ -223,7 +247,7 @@ struct Euler {
 #pragma unroll
       for (int k = 0; k < DIM; ++k) mm += u[1 + k] * u[1 + k];
       const R prho = (pp.gamma - R(1)) * (E * rho - R(0.5) * mm);   // p rho
-      const R r = R(1) / (prho * rho);
+      const R r = fast_rcp(prho * rho);
       const R ir = prho * r;                                         // 1 / rho
 #pragma unroll
       for (int k = 0; k < DIM; ++k) q[1 + k] = u[1 + k] * ir;
@@ -373,7 +397,7 @@ struct GlmMhd {
       // one FP64 division: p rho = (gamma-1)(rho (E - |B|^2/2 - psi^2/2) - |m|^2/2)
       const R mm = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
       const R prho = (pp.gamma - R(1)) * (rho * (u[4] - R(0.5) * BB - R(0.5) * psi * psi) - R(0.5) * mm);
-      const R r = R(1) / (prho * rho);
+      const R r = fast_rcp(prho * rho);
       ir = prho * r;
       p = prho * ir;
       irp = rho * rho * rho * r;
