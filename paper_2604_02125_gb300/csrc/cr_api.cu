@@ -125,18 +125,45 @@ bool get_ops(int eq, int dim, int prec, int vol, int N, VariantOps* o, int ncflu
   return false;
 }
 
-void fill_ref_tables(int N, const MeshArgs& ma, RefTab<double>* t64, RefTab<float>* t32) {
+void fill_ref_tables(int N, int eq, const MeshArgs& ma, RefTab<double>* t64, RefTab<float>* t32) {
   double xi[6], w[6], D[6][6];
   ref_tables(N, xi, w, D);
   std::memset(t64, 0, sizeof(*t64));
   std::memset(t32, 0, sizeof(*t32));
+  const double sa = eq == CR_EULER ? 2.0 : 0.5;   // row scale of the two-point flux (RefTab::A)
+  for (int d = 0; d < 4; ++d)
+    for (int p = 0; p <= N; ++p) {
+      const double sc = d < 3 ? ma.inv_dx[d] : 1.0;
+      for (int q = 0; q <= N; ++q) {
+        t64->B[d][p][q] = D[p][q] * sc;
+        t32->B[d][p][q] = (float)t64->B[d][p][q];
+      }
+      // The rows of D add up to zero (a uniform flux has no residual); rounded
+      // to FP32 they miss it by an ulp of their largest entry, which a large
+      // uniform pressure turns into the form's leading error.  The diagonal of
+      // the end rows, the smallest off-diagonal entry of an inner row (whose
+      // diagonal is zero), is taken as minus the sum of the others.
+      int m = p;
+      if (p > 0 && p < N) {
+        for (int q = 0; q <= N; ++q)
+          if (q != p && (m == p || std::fabs(D[p][q]) < std::fabs(D[p][m]))) m = q;
+        t32->B[d][p][p] = 0.0f;
+      }
+      double rest = 0.0;
+      for (int q = 0; q <= N; ++q)
+        if (q != m) rest += (double)t32->B[d][p][q];
+      t32->B[d][p][m] = (float)-rest;
+      for (int q = 0; q <= N; ++q) {
+        t64->A[d][p][q] = sa * t64->B[d][p][q];
+        t32->A[d][p][q] = (float)sa * t32->B[d][p][q];
+      }
+    }
   for (int p = 0; p < 6; ++p) {
     for (int q = 0; q < 6; ++q) {
-      t64->D[p][q] = (p <= N && q <= N) ? D[p][q] : 0.0;
-      t32->D[p][q] = (float)t64->D[p][q];
-      t32->D2f[p][q] = t64->D2f[p][q] = make_float2(2.0f * t32->D[p][q], 2.0f * t32->D[p][q]);
-      t32->D2s[p][q] = t64->D2s[p][q] =
-          make_float2(2.0f * t32->D[p][q] * ma.inv_dx_f[0], 2.0f * t32->D[p][q] * ma.inv_dx_f[1]);
+      t32->A2[0][p][q] = make_float2(t32->A[0][p][q], t32->A[1][p][q]);
+      t32->B2[0][p][q] = make_float2(t32->B[0][p][q], t32->B[1][p][q]);
+      t32->A2[1][p][q] = make_float2(t32->A[kTabPlain][p][q], t32->A[kTabPlain][p][q]);
+      t32->B2[1][p][q] = make_float2(t32->B[kTabPlain][p][q], t32->B[kTabPlain][p][q]);
     }
     t64->w[p] = t32->w[p] = p <= N ? w[p] : 0.0;
   }
@@ -220,9 +247,9 @@ void fill_launch_ctx(const cr_mesh_desc& d, const VariantOps& o, LaunchCtx* plc)
   lc.ma.dt_fixed = d.dt_fixed;
   lc.ma.gamma = d.gamma;
   lc.ma.c_h = d.c_h;
-  lc.pp64 = PhysParams<double>{d.gamma, 1.0 / (d.gamma - 1.0), d.c_h, d.vol};
-  lc.pp32 = PhysParams<float>{(float)d.gamma, (float)(1.0 / (d.gamma - 1.0)), (float)d.c_h, d.vol};
-  fill_ref_tables(d.degree_N, lc.ma, &lc.tb64, &lc.tb32);
+  lc.pp64 = make_phys<double>(d.gamma, d.c_h);
+  lc.pp32 = make_phys<float>(d.gamma, d.c_h);
+  fill_ref_tables(d.degree_N, d.eq, lc.ma, &lc.tb64, &lc.tb32);
   lc.epb = default_epb(o);
   int dev = 0;
   cudaGetDevice(&dev);

@@ -121,9 +121,9 @@ extern "C" int cr_step_noalloc(const cr_mesh_desc* desc, const double* u_in, dou
   lc.ma.dt_fixed = d.dt_fixed;
   lc.ma.gamma = d.gamma;
   lc.ma.c_h = d.c_h;
-  lc.pp64 = PhysParams<double>{d.gamma, 1.0 / (d.gamma - 1.0), d.c_h, d.vol};
-  lc.pp32 = PhysParams<float>{(float)d.gamma, (float)(1.0 / (d.gamma - 1.0)), (float)d.c_h, d.vol};
-  fill_ref_tables(d.degree_N, lc.ma, &lc.tb64, &lc.tb32);
+  lc.pp64 = make_phys<double>(d.gamma, d.c_h);
+  lc.pp32 = make_phys<float>(d.gamma, d.c_h);
+  fill_ref_tables(d.degree_N, d.eq, lc.ma, &lc.tb64, &lc.tb32);
   lc.epb = default_epb(o);
   lc.sms = 1;
   if ((e = cudaDeviceGetAttribute(&lc.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return to_status(e);

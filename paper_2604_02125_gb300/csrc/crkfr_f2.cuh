@@ -51,35 +51,38 @@ __device__ __forceinline__ f2& operator*=(f2& a, f2 b) { return a = f2(a * b); }
 
 __device__ __forceinline__ f2 fast_rcp(f2 x) { return f2(fast_rcp(x.v.x), fast_rcp(x.v.y)); }
 
+__device__ __forceinline__ f2 mad(f2 a, f2 b, f2 c) { return f2(__ffma2_rn(a.v, b.v, c.v)); }
+
 __device__ __forceinline__ f2 series_F(f2 u) {
-  const f2 c9(1.0f / 9.0f), c7(1.0f / 7.0f), c5(1.0f / 5.0f), c3(1.0f / 3.0f), c1(1.0f);
-  return u * (u * (u * (u * c9 + c7) + c5) + c3) + c1;
+  const f2 c3(0.15462606f), c2(0.19962572f), c1(0.33333710f), c0(1.0f);
+  return u * (u * (u * c3 + c2) + c1) + c0;
 }
 
-__device__ __forceinline__ f2 series_invF(f2 u) {
-  const f2 c4(-428.0f / 14175.0f), c3(-44.0f / 945.0f), c2(-4.0f / 45.0f), c1(-1.0f / 3.0f), c0(1.0f);
-  return u * (u * (u * (u * c4 + c3) + c2) + c1) + c0;
+__device__ __forceinline__ f2 series_invF4(f2 u) {   // 1/(4 F(u))
+  const f2 c3(-0.25f * 0.049737233f), c2(-0.25f * 0.088788078f), c1(-0.25f * 0.33333435f), c0(0.25f);
+  return u * (u * (u * c3 + c2) + c1) + c0;
 }
 
-// L(a1,b1) and 1/L(a2,b2) in both halves, as the scalar FP32 version: one
+// L(a1,b1)/2 and 1/(2 L(a2,b2)) in both halves, as the scalar FP32 version: one
 // reciprocal per half, one branch for all four series tests (the common
 // case), otherwise each half takes the scalar route.
-__device__ __forceinline__ void logmean_pair(f2 a1, f2 b1, f2 a2, f2 b2, f2& L1, f2& iL2) {
+__device__ __forceinline__ void logmean_pair(f2 a1, f2 b1, f2 a2, f2 b2, f2& H1, f2& T2, f2& rs2) {
   const f2 s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
   const f2 r = fast_rcp(f2(s1 * s2));
-  const f2 rs1 = s2 * r, rs2 = s1 * r;
+  const f2 rs1 = s2 * r;
+  rs2 = s1 * r;
   const f2 q1 = d1 * rs1, q2 = d2 * rs2;
   const f2 u1 = q1 * q1, u2 = q2 * q2;
   const float um = fmaxf(fmaxf(u1.v.x, u1.v.y), fmaxf(u2.v.x, u2.v.y));
   if (um < LogMeanEps<float>::v) {
-    L1 = f2(0.5f) * s1 * series_invF(u1);
-    iL2 = f2(2.0f) * series_F(u2) * rs2;
+    H1 = s1 * series_invF4(u1);
+    T2 = series_F(u2) * rs2;
   } else {
-    float l1x, l1y, i2x, i2y;
-    logmean_pair(a1.v.x, b1.v.x, a2.v.x, b2.v.x, l1x, i2x);
-    logmean_pair(a1.v.y, b1.v.y, a2.v.y, b2.v.y, l1y, i2y);
-    L1 = f2(l1x, l1y);
-    iL2 = f2(i2x, i2y);
+    float h1x, h1y, t2x, t2y, rx, ry;
+    logmean_pair(a1.v.x, b1.v.x, a2.v.x, b2.v.x, h1x, t2x, rx);
+    logmean_pair(a1.v.y, b1.v.y, a2.v.y, b2.v.y, h1y, t2y, ry);
+    H1 = f2(h1x, h1y);
+    T2 = f2(t2x, t2y);
   }
 }
 

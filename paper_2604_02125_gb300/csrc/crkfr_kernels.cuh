@@ -73,22 +73,31 @@ template <typename R> __device__ __forceinline__ R inv_dx_of(const MeshArgs& ma,
 template <> __device__ __forceinline__ double inv_dx_of<double>(const MeshArgs& ma, int d) { return ma.inv_dx[d]; }
 template <> __device__ __forceinline__ float inv_dx_of<float>(const MeshArgs& ma, int d) { return ma.inv_dx_f[d]; }
 
+// Coefficients of the flux differencing, D_pq = l_q'(xi_p) on [0,1].  A[d] and
+// B[d] carry 1/dx_d of a single solve (d < 3), so its residuals need no scaling
+// at the end of a line; A[3] and B[3] are without it (the batched kernels, which
+// share one table among solves of different sizes, scale).
+//   A: the pair coefficient of an unscaled row of the two-point flux, 2 D_pq
+//      (Euler) or D_pq / 2 (GLM-MHD, whose two-point flux comes out times 4)
+//   B: D_pq (rows scaled by two, the central flux, the non-conservative term)
+// FP32: A2, B2 as ready register pairs (x, y) of the packed FP32x2 pair loop,
+// [0] with 1/dx and 1/dy, [1] without (measured 53.8 -> 52.5 us per volume
+// launch, 2D Euler 256^2, N = 3, against forming the pairs in the loop, and
+// 52.7 -> 51.4 us for the folded 1/dx).
+constexpr int kTabPlain = 3;
 template <typename R>
-struct RefTab {
-  R D[6][6];       // D_pq = l_q'(xi_p) on [0,1]
+struct RefTabPairs {};
+template <>
+struct RefTabPairs<float> {
+  float2 A2[2][6][6], B2[2][6][6];
+};
+template <typename R>
+struct RefTab : RefTabPairs<R> {
+  R A[4][6][6], B[4][6][6];
   R iw0, iwN;      // 1/w_0, 1/w_N
   double w[6];     // quadrature weights (FP64, diagnostics)
   R a[7][7], b[7]; // Butcher tableau of the degree (same values as rk_a / rk_b)
   signed char slot[7];   // register slot of a stage residual needed beyond the next stage, else -1
-  // (2 D_pq, 2 D_pq) in FP32: the coefficients of the packed FP32x2 pair loop
-  // as ready register pairs (measured 53.8 -> 52.5 us per volume launch, 2D
-  // Euler 256^2, N = 3, against forming them from D_pq in the loop)
-  float2 D2f[6][6];
-  // (2 D_pq / dx, 2 D_pq / dy) of one solve: a single solve's packed pair loop
-  // folds the 1/dx scaling of its two lines into the coefficients (measured
-  // 52.7 -> 51.4 us per volume launch, 2D Euler 256^2, N = 3); the batched
-  // kernels, which share one table among solves of different sizes, scale
-  float2 D2s[6][6];
 };
 
 // Step record of one solve.  The CFL reduction needs no fence and no
@@ -276,6 +285,85 @@ __device__ __forceinline__ unsigned neighbour_of(unsigned e, const unsigned (&c)
   return c[d] == 0 ? e + (nd - 1) * stride : e - stride;
 }
 
+// Flux differencing along one line of n = N+1 nodes in direction d from the
+// pair data q: acc_p = (1/dx) (sum_q 2 D_pq f_S(q_p, q_q) [+ B(q_p) sum_q D_pq g(q_q)]).
+// Every pair is evaluated once (f_S is symmetric); D_pp f(q_p) only at the two
+// end points of a GLL line, where D_pp is non-zero.  The central flux,
+// (f(q_p) + f(q_q))/2, is differenced as sum_q D_pq f(q_q), the same sum since
+// the rows of D add up to zero.  fend: the physical fluxes at the two ends.
+// PRE: coefficients with 1/dx of direction td; else the plain ones, and the
+// result is scaled by inv_dx.
+template <class EQ, int N, typename R, bool PRE>
+__device__ __forceinline__ void line_differences(int d, const R (&q)[N + 1][EQ::P], R (&acc)[N + 1][EQ::M],
+                                                 R (&fend)[2][EQ::M], const PhysParams<R>& pp, const RefTab<R>& tb,
+                                                 int td, R inv_dx) {
+  constexpr int n = N + 1, M = EQ::M;
+  const R (&A)[6][6] = tb.A[PRE ? td : kTabPlain];
+  const R (&B)[6][6] = tb.B[PRE ? td : kTabPlain];
+  EQ::flux(d, q[0], fend[0], pp);
+  EQ::flux(d, q[N], fend[1], pp);
+  if constexpr (EQ::VOL == VOL_CENTRAL) {
+#pragma unroll
+    for (int a = 0; a < n; ++a)
+#pragma unroll
+      for (int v = 0; v < M; ++v) acc[a][v] = B[a][0] * fend[0][v] + B[a][N] * fend[1][v];
+#pragma unroll
+    for (int b = 1; b < N; ++b) {
+      R f[M];
+      EQ::flux(d, q[b], f, pp);
+#pragma unroll
+      for (int a = 0; a < n; ++a)
+        if (a != b)   // D_bb = 0 at the inner nodes
+#pragma unroll
+          for (int v = 0; v < M; ++v) acc[a][v] += B[a][b] * f[v];
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < n; ++k)
+#pragma unroll
+      for (int v = 0; v < M; ++v) acc[k][v] = R(0);
+    const R c0 = R(2) * B[0][0], cN = R(2) * B[N][N];
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      acc[0][v] = c0 * fend[0][v];
+      acc[N][v] = cN * fend[1][v];
+    }
+#pragma unroll
+    for (int a = 0; a < n; ++a)
+#pragma unroll
+      for (int b = a + 1; b < n; ++b) {
+        R f[M];
+        EQ::two_point(d, q[a], q[b], f, pp);
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          acc[a][v] += (EQ::half(v) ? B[a][b] : A[a][b]) * f[v];
+          acc[b][v] += (EQ::half(v) ? B[b][a] : A[b][a]) * f[v];
+        }
+      }
+  }
+  if constexpr (EQ::NC) {
+    // sum_q D_pq B(u_p) g(u_q) = B(u_p) (D g)_p (no factor 2)
+#pragma unroll
+    for (int a = 0; a < n; ++a) {
+      R dg[2] = {R(0), R(0)};
+#pragma unroll
+      for (int b = 0; b < n; ++b) {
+        R g[2];
+        EQ::ncg(d, q[b], g);
+        dg[0] += B[a][b] * g[0];
+        dg[1] += B[a][b] * g[1];
+      }
+      EQ::nc_apply(d, q[a], dg, acc[a]);
+    }
+  }
+  if constexpr (!PRE) {
+#pragma unroll
+    for (int k = 0; k < n; ++k)
+#pragma unroll
+      for (int v = 0; v < M; ++v) acc[k][v] *= inv_dx;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Volume kernel, tile form: one CTA holds epb elements; one thread per line.
 // Used where the lane form below does not fit in shared memory.
@@ -414,51 +502,12 @@ __device__ __forceinline__ void volume_tile_body(const double* __restrict__ u, R
 #pragma unroll
           for (int c = 0; c < P; ++c) q[k][c] = my[L::O_Q + c * NP + base + k * stride];
         R acc[n][M];
+        R fend[2][M];
+        line_differences<EQ, N, R, true>(d, q, acc, fend, pp, tb, d, R(1));
 #pragma unroll
         for (int k = 0; k < n; ++k)
 #pragma unroll
-          for (int v = 0; v < M; ++v) acc[k][v] = R(0);
-        // D_pp f(u_p): non-zero only at the two end points of a GLL line
-        {
-          R f[M];
-          EQ::flux(d, q[0], f, pp);
-#pragma unroll
-          for (int v = 0; v < M; ++v) acc[0][v] += R(2) * tb.D[0][0] * f[v];
-          EQ::flux(d, q[N], f, pp);
-#pragma unroll
-          for (int v = 0; v < M; ++v) acc[N][v] += R(2) * tb.D[N][N] * f[v];
-        }
-        // every pair once: f_S is symmetric
-#pragma unroll
-        for (int a = 0; a < n; ++a)
-#pragma unroll
-          for (int b = a + 1; b < n; ++b) {
-            R f[M];
-            EQ::two_point(d, q[a], q[b], f, pp);
-            const R dab = R(2) * tb.D[a][b], dba = R(2) * tb.D[b][a];
-#pragma unroll
-            for (int v = 0; v < M; ++v) { acc[a][v] += dab * f[v]; acc[b][v] += dba * f[v]; }
-          }
-        if constexpr (EQ::NC) {
-          // sum_q D_pq B(u_p) g(u_q) = B(u_p) (D g)_p (no factor 2)
-#pragma unroll
-          for (int a = 0; a < n; ++a) {
-            R dg[2] = {R(0), R(0)};
-#pragma unroll
-            for (int b = 0; b < n; ++b) {
-              R g[2];
-              EQ::ncg(d, q[b], g);
-              dg[0] += tb.D[a][b] * g[0];
-              dg[1] += tb.D[a][b] * g[1];
-            }
-            EQ::nc_apply(d, q[a], dg, acc[a]);
-          }
-        }
-        const R idx_d = inv_dx_of<R>(ma, d);
-#pragma unroll
-        for (int k = 0; k < n; ++k)
-#pragma unroll
-          for (int v = 0; v < M; ++v) my[L::O_RS + (i * M + v) * NP + base + k * stride] += acc[k][v] * idx_d;
+          for (int v = 0; v < M; ++v) my[L::O_RS + (i * M + v) * NP + base + k * stride] += acc[k][v];
       }
       __syncthreads();
     }
@@ -553,7 +602,8 @@ __device__ __forceinline__ void jump_of(const R* o, const R* x, int d, int side_
   // own is the '-' state when it is the xi = 1 side: U+ - U- = sgn (Ux - Uo)
   const R sgn = side_own == 1 ? R(1) : R(-1);
 #pragma unroll
-  for (int v = 0; v < M; ++v) J[v] = R(0.5) * (o[M + v] + x[M + v]) - R(0.5) * lam * sgn * (x[v] - o[v]) - o[M + v];
+  for (int v = 0; v < M; ++v)
+    J[v] = mad(R(0.5), o[M + v] + x[M + v], mulr(R(-0.5) * lam * sgn, x[v] - o[v])) - o[M + v];
   if constexpr (EQ::NC) {
     // + B(u^n_own) g^avg(U) - F^nc_own (the stage-wise flux adds its own sum
     // in face_jump instead of the first term)

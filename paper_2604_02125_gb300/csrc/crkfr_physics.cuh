@@ -23,8 +23,22 @@ __host__ __device__ constexpr int ipow(int b, int e) { return e == 0 ? 1 : b * i
 template <typename R>
 struct PhysParams {
   R gamma, inv_gm1, c_h;
-  int vol;
+  R inv4;   // 4 / (gamma - 1): the energy row of the scaled two-point fluxes
+  R ch2;    // 2 c_h
 };
+template <typename R>
+__host__ __device__ __forceinline__ PhysParams<R> make_phys(double gamma, double c_h) {
+  return PhysParams<R>{R(gamma), R(1.0 / (gamma - 1.0)), R(c_h), R(4.0 / (gamma - 1.0)), R(2.0 * c_h)};
+}
+
+// a b + c with one rounding, where a sum of two products would leave the choice
+// of the fused one to the compiler: every kernel that evaluates a flux then
+// rounds it the same way
+__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+// a product that is rounded by itself, never fused into a sum
+__device__ __forceinline__ double mulr(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b); }
 
 // ---------------------------------------------------------------------------
 // Logarithmic mean L(a,b) = (a-b)/(ln a - ln b) and its inverse.
@@ -35,8 +49,8 @@ struct PhysParams {
 // 50 digits; error below 9e-18), inside it degree 3 below u = 2^-13 (error
 // below 2e-19); above 1/16 the ratio a/b exceeds 1.66 and log(a/b) is well
 // conditioned (at u = 1e-4 the quotient's rounding costs log(a/b) 1e-16 / 0.02).
-// FP32: 5 terms below u = 0.05 (truncation below u^5 / (11 (1 - u)) < 3e-8,
-// half an FP32 ulp of F ~ 1); above it the ratio a/b exceeds 1.57.
+// FP32: degree 3 below u = 0.05 (least-maximum fits on [0, 0.05]; error below
+// 6.2e-9, a tenth of an FP32 ulp of F ~ 1); above it the ratio a/b exceeds 1.57.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double series_F(double u) {
   return 1.0 + u * (0.33333333333331369 + u * (0.20000000000836662 + u * (0.14285714148744664 + u * (0.11111122319976208
@@ -50,16 +64,17 @@ __device__ __forceinline__ double series_invF(double u) {
 __device__ __forceinline__ double series_F_near(double u) {
   return 1.0 + u * (0.33333333333338387 + u * (0.19999999793002216 + u * 0.14288427331899907));
 }
-__device__ __forceinline__ double series_invF_near(double u) {
-  return 1.0 + u * (-0.33333333333334706 + u * (-0.088888888326392527 + u * -0.046568219037031879));
+__device__ __forceinline__ double series_invF_near4(double u) {   // 1/(4 F(u))
+  return 0.25 + u * (-0.25 * 0.33333333333334706 + u * (-0.25 * 0.088888888326392527 + u * (-0.25 * 0.046568219037031879)));
 }
 __device__ __forceinline__ float series_F(float u) {
-  return 1.0f + u * (1.0f / 3.0f + u * (1.0f / 5.0f + u * (1.0f / 7.0f + u * (1.0f / 9.0f))));
+  return 1.0f + u * (0.33333710f + u * (0.19962572f + u * 0.15462606f));
 }
-// 1/F(u) by its own series (five terms; the truncation is below 7e-9 relative
-// for u < 0.05), so that the series branch needs a single reciprocal
 __device__ __forceinline__ float series_invF(float u) {
-  return 1.0f + u * (-1.0f / 3.0f + u * (-4.0f / 45.0f + u * (-44.0f / 945.0f + u * (-428.0f / 14175.0f))));
+  return 1.0f + u * (-0.33333435f + u * (-0.088788078f + u * -0.049737233f));
+}
+__device__ __forceinline__ float series_invF4(float u) {   // 1/(4 F(u))
+  return 0.25f + u * (-0.25f * 0.33333435f + u * (-0.25f * 0.088788078f + u * (-0.25f * 0.049737233f)));
 }
 template <typename R> struct LogMeanEps;
 template <> struct LogMeanEps<double> { static constexpr double v = 0.0625; };
@@ -106,32 +121,37 @@ __device__ __forceinline__ R inv_logmean(R a, R b) {
 // Out of line so that the compiler cannot if-convert it into the common path
 // (a predicated copy would be executed by every pair).
 template <typename R>
-__device__ __noinline__ void logmean_pair_general(R a1, R b1, R a2, R b2, R& L1, R& iL2) {
-  L1 = logmean(a1, b1);
-  iL2 = inv_logmean(a2, b2);
+__device__ __noinline__ void logmean_pair_general(R a1, R b1, R a2, R b2, R& H1, R& T2) {
+  H1 = R(0.5) * logmean(a1, b1);
+  T2 = R(0.5) * inv_logmean(a2, b2);
 }
 
-// L(a1,b1) and 1/L(a2,b2) together: one reciprocal, 1/(s1 s2), gives both 1/s1
-// and 1/s2, and one branch decides for both which form applies (the series on
-// resolved data; otherwise each takes its own branch above).
-__device__ __forceinline__ void logmean_pair(float a1, float b1, float a2, float b2, float& L1, float& iL2) {
+// Both logarithmic means of a pair in the scale the two-point fluxes take them
+// (powers of two folded into the polynomials or the callers' coefficients):
+// H1 = L(a1,b1) / 2 and T2 = 1 / (2 L(a2,b2)), and rs2 = 1/(a2 + b2).  One
+// reciprocal, 1/(s1 s2), gives both 1/s1 and 1/s2, and one branch decides for
+// both which form applies (the polynomials on resolved data; otherwise each
+// takes its own branch above).
+__device__ __forceinline__ void logmean_pair(float a1, float b1, float a2, float b2, float& H1, float& T2,
+                                             float& rs2) {
   const float s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
   const float r = fast_rcp(s1 * s2);
-  const float rs1 = s2 * r, rs2 = s1 * r;
+  const float rs1 = s2 * r;
+  rs2 = s1 * r;
   const float f1 = d1 * rs1, f2 = d2 * rs2;
   const float u1 = f1 * f1, u2 = f2 * f2;
   if (fmaxf(u1, u2) < LogMeanEps<float>::v) {
-    L1 = 0.5f * s1 * series_invF(u1);
-    iL2 = 2.0f * series_F(u2) * rs2;
+    H1 = s1 * series_invF4(u1);
+    T2 = series_F(u2) * rs2;
   } else {
-    logmean_pair_general(a1, b1, a2, b2, L1, iL2);
+    logmean_pair_general(a1, b1, a2, b2, H1, T2);
   }
 }
 
 // the wide polynomials of both means, out of line (twenty instructions on the
 // FP64 pipe that most pairs of a resolved flow do not need)
 static __device__ __noinline__ void series_pair_wide(double u1, double u2, double& g1, double& f2) {
-  g1 = series_invF(u1);
+  g1 = 0.25 * series_invF(u1);
   f2 = series_F(u2);
 }
 
@@ -143,25 +163,27 @@ static __device__ __noinline__ void series_pair_wide(double u1, double u2, doubl
 // divisions) instead of the wide polynomials, as a single bound of 1e-4 did,
 // took 124 against 71 us per volume launch on the 64-element 1D wave and 2138
 // against 1846 us on the shear layer (with the three-FMA reciprocal).
-__device__ __forceinline__ void logmean_pair(double a1, double b1, double a2, double b2, double& L1, double& iL2) {
+__device__ __forceinline__ void logmean_pair(double a1, double b1, double a2, double b2, double& H1, double& T2,
+                                             double& rs2) {
   const double s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
   const double r = fast_rcp(s1 * s2);
-  const double rs1 = s2 * r, rs2 = s1 * r;
+  const double rs1 = s2 * r;
+  rs2 = s1 * r;
   const double f1 = d1 * rs1, f2 = d2 * rs2;
   const double u1 = f1 * f1, u2 = f2 * f2;
   const unsigned h = max((unsigned)__double2hiint(u1), (unsigned)__double2hiint(u2));
   if (h < 0x3FB00000u) {   // 1/16
     double g, f;
     if (h < 0x3F200000u) {   // 2^-13
-      g = series_invF_near(u1);
+      g = series_invF_near4(u1);
       f = series_F_near(u2);
     } else {
       series_pair_wide(u1, u2, g, f);
     }
-    L1 = 0.5 * s1 * g;
-    iL2 = 2.0 * f * rs2;
+    H1 = s1 * g;
+    T2 = f * rs2;
   } else {
-    logmean_pair_general(a1, b1, a2, b2, L1, iL2);
+    logmean_pair_general(a1, b1, a2, b2, H1, T2);
   }
 }
 
@@ -277,7 +299,7 @@ struct Euler {
       R ke = R(0);
 #pragma unroll
       for (int k = 0; k < DIM; ++k) ke += q[1 + k] * q[1 + k];
-      return q[IP] * pp.inv_gm1 + R(0.5) * q[0] * ke;
+      return mad(q[IP], pp.inv_gm1, R(0.5) * q[0] * ke);
     }
     return q[0] * q[IAUX];
   }
@@ -301,42 +323,51 @@ struct Euler {
     f[DIM + 1] = q[1 + d] * (total_energy(q, pp) + q[IP]);
   }
 
-  // symmetric two-point flux f_S(q_a, q_b) in direction d
+  // Symmetric two-point flux f_S(q_a, q_b) in direction d, scaled so that sums
+  // stand in for means: f_S,v = f[v] / 2 where half(v), else f[v]; the
+  // differentiation coefficients, D_pq and 2 D_pq, carry the factor, so no
+  // instruction multiplies by one half.  Kennedy-Gruber: every row halved,
+  // with one addition more -- with two coefficients per pair the front end of
+  // the compiler (CUDA 13.0, its optimisation levels above 1) miscompiled the
+  // branch-free FP32 pair loops of degree 4 and 5 (a constant state lost a
+  // fifth of its mass in a step; the per-variant tests caught it).
+  __host__ __device__ static constexpr bool half(int v) { return VOL == VOL_KEP || v > 0; }
   template <typename R>
   __device__ __forceinline__ static void two_point(int d, const R* a, const R* b, R* f, const PhysParams<R>& pp) {
-    R vavg[DIM];
+    static_assert(VOL != VOL_CENTRAL, "the central flux is differenced as sum_q D_pq f(q_q)");
+    R vs[DIM];
 #pragma unroll
-    for (int k = 0; k < DIM; ++k) vavg[k] = R(0.5) * (a[1 + k] + b[1 + k]);
-    R pavg = R(0.5) * (a[IP] + b[IP]);
+    for (int k = 0; k < DIM; ++k) vs[k] = a[1 + k] + b[1 + k];
+    const R ps = a[IP] + b[IP];
     if constexpr (VOL == VOL_EC) {
       // Ranocha: rho^ln {{v}}, momentum f_rho {{v}} + {{p}} n, energy with
       // 1/ln-mean(rho/p) and the product p_a v_b + p_b v_a
-      R rho_ln, irp_ln;
-      logmean_pair(a[0], b[0], a[IAUX], b[IAUX], rho_ln, irp_ln);
-      R f0 = rho_ln * vavg[d];
-      R vv = R(0);
+      R h, t, rs;
+      logmean_pair(a[0], b[0], a[IAUX], b[IAUX], h, t, rs);
+      const R f0 = h * vs[d];
+      R w = pp.inv4 * t;
 #pragma unroll
-      for (int k = 0; k < DIM; ++k) vv += a[1 + k] * b[1 + k];
+      for (int k = 0; k < DIM; ++k) w = mad(a[1 + k], b[1 + k], w);
       f[0] = f0;
 #pragma unroll
-      for (int k = 0; k < DIM; ++k) f[1 + k] = f0 * vavg[k] + (k == d ? pavg : R(0));
-      f[DIM + 1] = f0 * (R(0.5) * vv + pp.inv_gm1 * irp_ln)
-                 + R(0.5) * (a[IP] * b[1 + d] + b[IP] * a[1 + d]);
-    } else if constexpr (VOL == VOL_KEP) {
-      // Kennedy-Gruber: arithmetic means of rho, v, p and e = E/rho
-      R ravg = R(0.5) * (a[0] + b[0]);
-      R eavg = R(0.5) * (a[IAUX] + b[IAUX]);
-      R f0 = ravg * vavg[d];
-      f[0] = f0;
-#pragma unroll
-      for (int k = 0; k < DIM; ++k) f[1 + k] = f0 * vavg[k] + (k == d ? pavg : R(0));
-      f[DIM + 1] = (ravg * eavg + pavg) * vavg[d];
+      for (int k = 0; k < DIM; ++k) {
+        if (k == d) f[1 + k] = mad(f0, vs[k], ps);
+        else f[1 + k] = f0 * vs[k];
+      }
+      const R pv = a[IP] * b[1 + d];
+      f[DIM + 1] = mad(f0, w, mad(b[IP], a[1 + d], pv));
     } else {
-      R fa[M], fb[M];
-      flux(d, a, fa, pp);
-      flux(d, b, fb, pp);
+      // Kennedy-Gruber: arithmetic means of rho, v, p and e = E/rho
+      const R rq = R(0.25) * (a[0] + b[0]);
+      const R f0 = rq * vs[d];
+      f[0] = f0 + f0;
 #pragma unroll
-      for (int m = 0; m < M; ++m) f[m] = R(0.5) * (fa[m] + fb[m]);
+      for (int k = 0; k < DIM; ++k) {
+        if (k == d) f[1 + k] = mad(f0, vs[k], ps);
+        else f[1 + k] = f0 * vs[k];
+      }
+      // 2 (rho e + p) v = (rq (e_a + e_b) + ps / 2) vs
+      f[DIM + 1] = mad(rq, a[IAUX] + b[IAUX], R(0.5) * ps) * vs[d];
     }
   }
 
@@ -442,42 +473,49 @@ struct GlmMhd {
 
   // entropy-conservative flux: satisfies [[w]].f = [[psi_d]] + {{theta}} [[B_d]]
   // with theta = w.phi_Powell = rho (v.B)/p (derived from the entropy
-  // variables of S = -rho s/(gamma-1)); central flux for CR_VOL_CENTRAL.
+  // variables of S = -rho s/(gamma-1)).  Scaled so that sums stand in for
+  // means: f_S = f / 4 in every row, so the coefficient of the pair is D_pq / 2.
+  __host__ __device__ static constexpr bool half(int) { return false; }
   template <typename R>
   __device__ __forceinline__ static void two_point(int d, const R* a, const R* b, R* f, const PhysParams<R>& pp) {
-    if constexpr (VOL != VOL_EC) {
-      R fa[M], fb[M];
-      flux(d, a, fa, pp);
-      flux(d, b, fb, pp);
+    static_assert(VOL == VOL_EC, "the central flux is differenced as sum_q D_pq f(q_q)");
+    R v[3], B[3];   // sums of both nodes
 #pragma unroll
-      for (int m = 0; m < M; ++m) f[m] = R(0.5) * (fa[m] + fb[m]);
-      return;
+    for (int k = 0; k < 3; ++k) { v[k] = a[1 + k] + b[1 + k]; B[k] = a[IB + k] + b[IB + k]; }
+    const R psi = a[IPSI] + b[IPSI];
+    R h, t, rs2;
+    logmean_pair(a[0], b[0], a[IBETA], b[IBETA], h, t, rs2);
+    const R Bd = B[d];
+    const R f0 = h * v[d];              // rho^ln {{v_d}}
+    const R g0 = f0 + f0;
+    f[0] = g0 + g0;
+    // 4 (p~ + {{|B|^2}}/2), p~ = {{rho}} / (2 {{beta}})
+    const R rs = a[0] + b[0];
+    const R pt = mad(rs + rs, rs2, a[IB2] + b[IB2]);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const R m = k == d ? mad(g0, v[k], pt) : R(g0 * v[k]);
+      f[1 + k] = mad(-Bd, B[k], m);
     }
-    R v[3], B[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) { v[k] = R(0.5) * (a[1 + k] + b[1 + k]); B[k] = R(0.5) * (a[IB + k] + b[IB + k]); }
-    R psi = R(0.5) * (a[IPSI] + b[IPSI]);
-    R rho_ln, ibeta_ln;
-    logmean_pair(a[0], b[0], a[IBETA], b[IBETA], rho_ln, ibeta_ln);
-    R ptil = (a[0] + b[0]) * fast_rcp(R(2) * (a[IBETA] + b[IBETA]));     // {{rho}} / (2 {{beta}})
-    R v2avg = R(0.5) * (a[IV2] + b[IV2]);
-    R B2avg = R(0.5) * (a[IB2] + b[IB2]);
-    R vB2avg = R(0.5) * (a[1 + d] * a[IB2] + b[1 + d] * b[IB2]);
-    R psiBavg = R(0.5) * (a[IPSI] * a[IB + d] + b[IPSI] * b[IB + d]);
-    R vBavg = R(0.5) * (a[IVB] + b[IVB]);
-    R Bd = B[d];
-    R ch = pp.c_h;
-    R f0 = rho_ln * v[d];
-    f[0] = f0;
+    for (int k = 0; k < 3; ++k) {
+      if (k == d) f[5 + k] = pp.ch2 * psi;
+      else f[5 + k] = mad(v[d], B[k], R(-(v[k] * Bd)));
+    }
+    f[8] = pp.ch2 * Bd;
+    // 8 f_E = e + 2 z
+    R z = Bd * (a[IVB] + b[IVB]);
+    z = mad(-a[1 + d], a[IB2], z);
+    z = mad(-b[1 + d], b[IB2], z);
+    const R pb = a[IPSI] * a[IB + d];
+    z = mad(-pp.ch2, mad(b[IPSI], b[IB + d], pb), z);
+    R e = g0 * mad(pp.inv4, t, -(a[IV2] + b[IV2]));
 #pragma unroll
-    for (int k = 0; k < 3; ++k) f[1 + k] = f0 * v[k] - Bd * B[k] + (k == d ? ptil + R(0.5) * B2avg : R(0));
-#pragma unroll
-    for (int k = 0; k < 3; ++k) f[5 + k] = (k == d) ? ch * psi : v[d] * B[k] - v[k] * Bd;
-    f[8] = ch * Bd;
-    f[4] = f0 * R(0.5) * (pp.inv_gm1 * ibeta_ln - v2avg)
-         + f[1] * v[0] + f[2] * v[1] + f[3] * v[2]
-         + f[5] * B[0] + f[6] * B[1] + f[7] * B[2] + f[8] * psi
-         - R(0.5) * vB2avg - ch * psiBavg + Bd * vBavg;
+    for (int k = 0; k < 3; ++k) {
+      e = mad(f[1 + k], v[k], e);
+      e = mad(f[5 + k], B[k], e);
+    }
+    f[4] = mad(R(0.5), mad(f[8], psi, e), z);
   }
 
   // |v_d| + max(c_f, c_h): the GLM pair travels at v_d -+ c_h

@@ -48,58 +48,6 @@ __host__ __device__ constexpr int rk_slot(int N, int j) {
 }
 __host__ __device__ constexpr int rk_nsaved(int N) { return rk_slot(N, rk_stages(N)); }
 
-// Flux differencing along one line of n = N+1 nodes in direction D from the
-// pair data q: acc_p = inv_dx (sum_q 2 D_pq f_S(q_p, q_q) [+ B(q_p) sum_q D_pq g(q_q)]).
-// Every pair is evaluated once (f_S is symmetric); D_pp f(q_p) only at the two
-// end points of a GLL line, where D_pp is non-zero.
-template <class EQ, int N, typename R, int D>
-__device__ __forceinline__ void line_residual(const R (&q)[N + 1][EQ::P], R (&acc)[N + 1][EQ::M],
-                                              R (&fend)[2][EQ::M], const PhysParams<R>& pp, const RefTab<R>& tb,
-                                              R inv_dx) {
-  constexpr int n = N + 1, M = EQ::M;
-#pragma unroll
-  for (int k = 0; k < n; ++k)
-#pragma unroll
-    for (int v = 0; v < M; ++v) acc[k][v] = R(0);
-  // physical fluxes at the two end points: the D_pp terms here, and the face
-  // sums of the time-averaged flux (eq. disc.avg.flux) in the caller
-  EQ::flux(D, q[0], fend[0], pp);
-  EQ::flux(D, q[N], fend[1], pp);
-#pragma unroll
-  for (int v = 0; v < M; ++v) {
-    acc[0][v] = R(2) * tb.D[0][0] * fend[0][v];
-    acc[N][v] = R(2) * tb.D[N][N] * fend[1][v];
-  }
-#pragma unroll
-  for (int a = 0; a < n; ++a)
-#pragma unroll
-    for (int b = a + 1; b < n; ++b) {
-      R f[M];
-      EQ::two_point(D, q[a], q[b], f, pp);
-      const R dab = R(2) * tb.D[a][b], dba = R(2) * tb.D[b][a];
-#pragma unroll
-      for (int v = 0; v < M; ++v) { acc[a][v] += dab * f[v]; acc[b][v] += dba * f[v]; }
-    }
-  if constexpr (EQ::NC) {
-#pragma unroll
-    for (int a = 0; a < n; ++a) {
-      R dg[2] = {R(0), R(0)};
-#pragma unroll
-      for (int b = 0; b < n; ++b) {
-        R g[2];
-        EQ::ncg(D, q[b], g);
-        dg[0] += tb.D[a][b] * g[0];
-        dg[1] += tb.D[a][b] * g[1];
-      }
-      EQ::nc_apply(D, q[a], dg, acc[a]);
-    }
-  }
-#pragma unroll
-  for (int k = 0; k < n; ++k)
-#pragma unroll
-    for (int v = 0; v < M; ++v) acc[k][v] *= inv_dx;
-}
-
 // The x-line and the y-line of one thread in the two halves of packed FP32
 // pairs (2D Euler, FP32 form).  Both lines are flux-differenced in a frame
 // rotated to the line: the y half holds (rho, v_y, v_x, p, aux), so the
@@ -122,34 +70,61 @@ __host__ __device__ constexpr int swap_xy(int c) {
   return c == 1 ? 2 : c == 2 ? 1 : (EQ::NC && c == 5) ? 6 : (EQ::NC && c == 6) ? 5 : c;
 }
 
-// PRE: the coefficients carry 1/dx of each line (RefTab::D2s), else the
-// residual is scaled at the end
+// PRE: the coefficients carry 1/dx of each line, else the residual is scaled
+// at the end
 template <class EQ, int N, bool PRE>
 __device__ __forceinline__ void line_residual_xy(const f2 (&q)[N + 1][EQ::P], f2 (&acc)[N + 1][EQ::M],
                                                  f2 (&fend)[2][EQ::M], const PhysParams<f2>& pp,
                                                  const RefTab<float>& tb, f2 inv_dx) {
   constexpr int n = N + 1, M = EQ::M;
+  const float2 (&A)[6][6] = tb.A2[PRE ? 0 : 1];
+  const float2 (&B)[6][6] = tb.B2[PRE ? 0 : 1];
 #pragma unroll
   for (int k = 0; k < n; ++k)
 #pragma unroll
     for (int v = 0; v < M; ++v) acc[k][v] = f2(0.0f);
+  if constexpr (EQ::VOL == VOL_CENTRAL) {
+    // sum_q D_pq f(q_q) (line_differences), D_bb = 0 at the inner nodes
 #pragma unroll
-  for (int a = 0; a < n; ++a)
-#pragma unroll
-    for (int b = a + 1; b < n; ++b) {
+    for (int b = 1; b < N; ++b) {
       f2 f[M];
-      EQ::two_point(0, q[a], q[b], f, pp);
-      const f2 dab(PRE ? tb.D2s[a][b] : tb.D2f[a][b]), dba(PRE ? tb.D2s[b][a] : tb.D2f[b][a]);
+      EQ::flux(0, q[b], f, pp);
 #pragma unroll
-      for (int v = 0; v < M; ++v) { acc[a][v] += dab * f[v]; acc[b][v] += dba * f[v]; }
+      for (int a = 0; a < n; ++a)
+        if (a != b)
+#pragma unroll
+          for (int v = 0; v < M; ++v) acc[a][v] += f2(B[a][b]) * f[v];
     }
-  // end points last: the fluxes there stay live only until the face sums
-  EQ::flux(0, q[0], fend[0], pp);
-  EQ::flux(0, q[N], fend[1], pp);
+    EQ::flux(0, q[0], fend[0], pp);
+    EQ::flux(0, q[N], fend[1], pp);
 #pragma unroll
-  for (int v = 0; v < M; ++v) {
-    acc[0][v] += f2(PRE ? tb.D2s[0][0] : tb.D2f[0][0]) * fend[0][v];
-    acc[N][v] += f2(PRE ? tb.D2s[N][N] : tb.D2f[N][N]) * fend[1][v];
+    for (int a = 0; a < n; ++a)
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        acc[a][v] += f2(B[a][0]) * fend[0][v];
+        acc[a][v] += f2(B[a][N]) * fend[1][v];
+      }
+  } else {
+#pragma unroll
+    for (int a = 0; a < n; ++a)
+#pragma unroll
+      for (int b = a + 1; b < n; ++b) {
+        f2 f[M];
+        EQ::two_point(0, q[a], q[b], f, pp);
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          acc[a][v] += f2(EQ::half(v) ? B[a][b] : A[a][b]) * f[v];
+          acc[b][v] += f2(EQ::half(v) ? B[b][a] : A[b][a]) * f[v];
+        }
+      }
+    // end points last: the fluxes there stay live only until the face sums
+    EQ::flux(0, q[0], fend[0], pp);
+    EQ::flux(0, q[N], fend[1], pp);
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      acc[0][v] += f2(A[0][0]) * fend[0][v];
+      acc[N][v] += f2(A[N][N]) * fend[1][v];
+    }
   }
   if constexpr (!PRE) {
 #pragma unroll
@@ -159,18 +134,19 @@ __device__ __forceinline__ void line_residual_xy(const f2 (&q)[N + 1][EQ::P], f2
   }
 }
 
-
 // Flux differencing of one line of the element at `my`, rolled over the pairs
 // so that the two-point flux is compiled once: pair data read from shared
 // memory (Q, component c at Q[c * NP + node]) in the frame of swap_xy when
-// sw is set, the residual (times inv_dx) added into shared memory (RY, in the
+// sw is set, the residual (coefficients with 1/dx of direction td) added into shared memory (RY, in the
 // element's own frame); the end nodes' pair data and fluxes are returned for
 // the face sums.  Every node of the line belongs to the calling thread.
 template <class EQ, int N, typename R>
 __device__ __forceinline__ void line_residual_rolled(const R* __restrict__ Q, R* __restrict__ RY, int NPv, int base,
                                                      int stride, bool sw, R (&qe)[N + 1][EQ::P], R (&fend)[2][EQ::M],
-                                                     const PhysParams<R>& pp, const RefTab<R>& tb, R inv_dx) {
+                                                     const PhysParams<R>& pp, const RefTab<R>& tb, int td) {
   constexpr int n = N + 1, M = EQ::M, P = EQ::P;
+  const R (&A)[6][6] = tb.A[td];
+  const R (&B)[6][6] = tb.B[td];
   auto load = [&](int node, R* q) {
 #pragma unroll
     for (int c = 0; c < P; ++c) q[c] = Q[(sw ? swap_xy<EQ>(c) : c) * NPv + node];
@@ -184,21 +160,34 @@ __device__ __forceinline__ void line_residual_rolled(const R* __restrict__ Q, R*
     const int na = base + a * stride;
     R qa[P], acc[M];
     load(na, qa);
-    // D_aa f(q_a): non-zero only at the two end points of a GLL line
-    const R caa = R(2) * tb.D[a][a] * inv_dx;
+    // D_aa f(q_a): non-zero only at the two end points of a GLL line; the
+    // central flux is differenced as sum_b D_ab f(q_b)
+    const R caa = (EQ::VOL == VOL_CENTRAL ? R(1) : R(2)) * B[a][a];
 #pragma unroll
     for (int v = 0; v < M; ++v) acc[v] = a == 0 ? caa * fend[0][v] : (a == N ? caa * fend[1][v] : R(0));
+    if constexpr (EQ::VOL == VOL_CENTRAL) {
 #pragma unroll 1
-    for (int b = a + 1; b < n; ++b) {
-      const int nb = base + b * stride;
-      R qb[P], f[M];
-      load(nb, qb);
-      EQ::two_point(0, qa, qb, f, pp);
-      const R cab = R(2) * tb.D[a][b] * inv_dx, cba = R(2) * tb.D[b][a] * inv_dx;
+      for (int b = 0; b < n; ++b) {
+        if (b == a) continue;
+        R qb[P], f[M];
+        load(base + b * stride, qb);
+        EQ::flux(0, qb, f, pp);
+        const R cab = B[a][b];
 #pragma unroll
-      for (int v = 0; v < M; ++v) {
-        acc[v] += cab * f[v];
-        RY[(sw ? swap_xy<EQ>(v) : v) * NPv + nb] += cba * f[v];
+        for (int v = 0; v < M; ++v) acc[v] += cab * f[v];
+      }
+    } else {
+#pragma unroll 1
+      for (int b = a + 1; b < n; ++b) {
+        const int nb = base + b * stride;
+        R qb[P], f[M];
+        load(nb, qb);
+        EQ::two_point(0, qa, qb, f, pp);
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          acc[v] += (EQ::half(v) ? B[a][b] : A[a][b]) * f[v];
+          RY[(sw ? swap_xy<EQ>(v) : v) * NPv + nb] += (EQ::half(v) ? B[b][a] : A[b][a]) * f[v];
+        }
       }
     }
     if constexpr (EQ::NC) {
@@ -207,7 +196,7 @@ __device__ __forceinline__ void line_residual_rolled(const R* __restrict__ Q, R*
 #pragma unroll 1
       for (int b = 0; b < n; ++b) {
         const int nb = base + b * stride;
-        const R dab = tb.D[a][b] * inv_dx;
+        const R dab = B[a][b];
         dg[0] += dab * Q[(sw ? swap_xy<EQ>(EQ::IB) : EQ::IB) * NPv + nb];
         dg[1] += dab * Q[EQ::IPSI * NPv + nb];
       }
@@ -407,8 +396,8 @@ __device__ __forceinline__ void issue_prefetch(const Prefetch& pf) {
 // [var][32][NP] (the tile's slice of the global layout).  S1 = 1: a single
 // stage with b = 1 (R-bar = R(u), face records of u), the volume part of one
 // stage of the multi-stage RKFR step.
-// PRE: a single solve's reference table (the packed pair loop's coefficients
-// carry 1/dx, RefTab::D2s); false for the batched kernels
+// PRE: a single solve's reference table (the flux-differencing coefficients
+// carry 1/dx); false for the batched kernels
 template <class EQ, int N, typename R, int SH = 0, int S1 = 0, bool PRE = false>
 __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, R* __restrict__ rbar,
                                                   R* __restrict__ trace, const DevState* __restrict__ st,
@@ -443,7 +432,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
   const bool active = el < nel;
   R* my = sm + (size_t)el * L::SZ;
   constexpr bool PACK = L::PACK;
-  const PhysParams<f2> pp2{f2(float(pp.gamma)), f2(float(pp.inv_gm1)), f2(float(pp.c_h)), pp.vol};
+  const PhysParams<f2> pp2{f2(float(pp.gamma)), f2(float(pp.inv_gm1)), f2(float(pp.c_h)), f2(float(pp.inv4)), f2(float(pp.ch2))};
 
   // ---- u^n: coalesced into shared memory (staging in the Q region), then own x-line to registers
   // (index arithmetic with compile-time divisors only).  FP32 form: the hardware conversion, one
@@ -543,7 +532,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
       // (packed form: together with the y-line below)
       if constexpr (!PACK && !ONEQ) {
         R fend[2][M];
-        line_residual<EQ, N, R, 0>(q, ax, fend, pp, tb, inv_dx_of<R>(ma, 0));
+        line_differences<EQ, N, R, PRE>(0, q, ax, fend, pp, tb, 0, inv_dx_of<R>(ma, 0));
         face_accumulate<EQ, N, R, 0>(fx, q, fend, bi, i == 0, pp);
       }
     }
@@ -586,7 +575,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
         if (active) {
           R qe[n][P], fe[2][M];
           line_residual_rolled<EQ, N, R>(my + L::O_Q, my + L::O_RY, NP, dir ? l : l * n, dir ? n : 1, dir != 0, qe,
-                                         fe, pp, tb, dir ? inv_dx_of<R>(ma, 1) : inv_dx_of<R>(ma, 0));
+                                         fe, pp, tb, dir);
           if (dir == 0) face_accumulate<EQ, N, R, 0>(fx, qe, fe, bi, i == 0, pp);
           else face_accumulate<EQ, N, R, 0>(fy, qe, fe, bi, i == 0, pp);   // swapped frame
         }
@@ -606,7 +595,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           for (int k = 0; k < n; ++k)
 #pragma unroll
             for (int c = 0; c < P; ++c) qd[k][c] = my[L::O_Q + (dir ? swap_xy<EQ>(c) : c) * NP + base + k * stride];
-          line_residual<EQ, N, R, 0>(qd, ad, fe, pp, tb, dir ? inv_dx_of<R>(ma, 1) : inv_dx_of<R>(ma, 0));
+          line_differences<EQ, N, R, PRE>(0, qd, ad, fe, pp, tb, dir, dir ? inv_dx_of<R>(ma, 1) : inv_dx_of<R>(ma, 0));
           if (dir == 0) {
 #pragma unroll
             for (int k = 0; k < n; ++k)
@@ -639,7 +628,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           write_stage_prims<EQ, N, R>(trace, 1, 0, l, i, E, e0 + el, qy[0]);
           write_stage_prims<EQ, N, R>(trace, 1, 1, l, i, E, e0 + el, qy[N]);
         }
-        line_residual<EQ, N, R, (DIM > 1 ? 1 : 0)>(qy, ay, fend, pp, tb, inv_dx_of<R>(ma, 1));
+        line_differences<EQ, N, R, PRE>(DIM > 1 ? 1 : 0, qy, ay, fend, pp, tb, 1, inv_dx_of<R>(ma, 1));
         face_accumulate<EQ, N, R, (DIM > 1 ? 1 : 0)>(fy, qy, fend, bi, i == 0, pp);
 #pragma unroll
         for (int k = 0; k < n; ++k)
@@ -656,7 +645,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           for (int k = 0; k < n; ++k)
 #pragma unroll
             for (int c = 0; c < P; ++c) qz[k][c] = my[L::O_Q + c * NP + base + k * n * n];
-          line_residual<EQ, N, R, DIM - 1>(qz, az, fend, pp, tb, inv_dx_of<R>(ma, DIM - 1));
+          line_differences<EQ, N, R, PRE>(DIM - 1, qz, az, fend, pp, tb, 2, inv_dx_of<R>(ma, DIM - 1));
           face_accumulate<EQ, N, R, DIM - 1>(fz, qz, fend, bi, i == 0, pp);
 #pragma unroll
           for (int k = 0; k < n; ++k)
@@ -1028,12 +1017,12 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
 #pragma unroll
     for (int k = 0; k < n; ++k)
 #pragma unroll
-      for (int v = 0; v < M; ++v) du[k][v] = -dtR * rb[v][k];
+      for (int v = 0; v < M; ++v) du[k][v] = mulr(-dtR, rb[v][k]);
     {
       // - dt J^- g_R'(1)/dx + dt J^+ (-g_L'(0))/dx at the x faces
       const R sR = dtR * tb.iwN * inv_dx_of<R>(ma, 0), sL = dtR * tb.iw0 * inv_dx_of<R>(ma, 0);
 #pragma unroll
-      for (int v = 0; v < M; ++v) { du[N][v] -= sR * Jm[v]; du[0][v] += sL * Jp[v]; }
+      for (int v = 0; v < M; ++v) { du[N][v] = mad(-sR, Jm[v], du[N][v]); du[0][v] = mad(sL, Jp[v], du[0][v]); }
     }
     // y / z faces: whole lines on the face (warp-uniform), scaled jumps from phase A
 #pragma unroll
