@@ -134,79 +134,6 @@ __device__ __forceinline__ void line_residual_xy(const f2 (&q)[N + 1][EQ::P], f2
   }
 }
 
-// Flux differencing of one line of the element at `my`, rolled over the pairs
-// so that the two-point flux is compiled once: pair data read from shared
-// memory (Q, component c at Q[c * NP + node]) in the frame of swap_xy when
-// sw is set, the residual (coefficients with 1/dx of direction td) added into shared memory (RY, in the
-// element's own frame); the end nodes' pair data and fluxes are returned for
-// the face sums.  Every node of the line belongs to the calling thread.
-template <class EQ, int N, typename R>
-__device__ __forceinline__ void line_residual_rolled(const R* __restrict__ Q, R* __restrict__ RY, int NPv, int base,
-                                                     int stride, bool sw, R (&qe)[N + 1][EQ::P], R (&fend)[2][EQ::M],
-                                                     const PhysParams<R>& pp, const RefTab<R>& tb, int td) {
-  constexpr int n = N + 1, M = EQ::M, P = EQ::P;
-  const R (&A)[6][6] = tb.A[td];
-  const R (&B)[6][6] = tb.B[td];
-  auto load = [&](int node, R* q) {
-#pragma unroll
-    for (int c = 0; c < P; ++c) q[c] = Q[(sw ? swap_xy<EQ>(c) : c) * NPv + node];
-  };
-  load(base, qe[0]);
-  load(base + N * stride, qe[N]);
-  EQ::flux(0, qe[0], fend[0], pp);
-  EQ::flux(0, qe[N], fend[1], pp);
-#pragma unroll 1
-  for (int a = 0; a < n; ++a) {
-    const int na = base + a * stride;
-    R qa[P], acc[M];
-    load(na, qa);
-    // D_aa f(q_a): non-zero only at the two end points of a GLL line; the
-    // central flux is differenced as sum_b D_ab f(q_b)
-    const R caa = (EQ::VOL == VOL_CENTRAL ? R(1) : R(2)) * B[a][a];
-#pragma unroll
-    for (int v = 0; v < M; ++v) acc[v] = a == 0 ? caa * fend[0][v] : (a == N ? caa * fend[1][v] : R(0));
-    if constexpr (EQ::VOL == VOL_CENTRAL) {
-#pragma unroll 1
-      for (int b = 0; b < n; ++b) {
-        if (b == a) continue;
-        R qb[P], f[M];
-        load(base + b * stride, qb);
-        EQ::flux(0, qb, f, pp);
-        const R cab = B[a][b];
-#pragma unroll
-        for (int v = 0; v < M; ++v) acc[v] += cab * f[v];
-      }
-    } else {
-#pragma unroll 1
-      for (int b = a + 1; b < n; ++b) {
-        const int nb = base + b * stride;
-        R qb[P], f[M];
-        load(nb, qb);
-        EQ::two_point(0, qa, qb, f, pp);
-#pragma unroll
-        for (int v = 0; v < M; ++v) {
-          acc[v] += (EQ::half(v) ? B[a][b] : A[a][b]) * f[v];
-          RY[(sw ? swap_xy<EQ>(v) : v) * NPv + nb] += (EQ::half(v) ? B[b][a] : A[b][a]) * f[v];
-        }
-      }
-    }
-    if constexpr (EQ::NC) {
-      // sum_b D_ab B(u_a) g(u_b) = B(u_a) (D g)_a (no factor 2)
-      R dg[2] = {R(0), R(0)};
-#pragma unroll 1
-      for (int b = 0; b < n; ++b) {
-        const int nb = base + b * stride;
-        const R dab = B[a][b];
-        dg[0] += dab * Q[(sw ? swap_xy<EQ>(EQ::IB) : EQ::IB) * NPv + nb];
-        dg[1] += dab * Q[EQ::IPSI * NPv + nb];
-      }
-      EQ::nc_apply(0, qa, dg, acc);
-    }
-#pragma unroll
-    for (int v = 0; v < M; ++v) RY[(sw ? swap_xy<EQ>(v) : v) * NPv + na] += acc[v];
-  }
-}
-
 // Time averages at the two end points of one line in direction D (the face
 // nodes of the two faces normal to D): U = sum_i b_i u^(i), F^D = sum_i b_i
 // f^D(u^(i)) (eq. disc.avg.flux), lambda_D(u^n), and for the non-conservative
@@ -225,27 +152,27 @@ struct FaceAcc : FaceAccNc<EQ, R> {
 };
 
 // Register budget of the 2D Euler lane kernels of degree 4 and 5 (resident
-// CTAs per SM; measured: more CTAs outweigh the spills up to the shared-memory
-// limit) and the highest degree that takes the packed x/y form.  Degree 4
-// packed runs at 2 CTAs per SM (168 registers, 108 B of spills): 99 against
-// 117 us per volume launch of the scalar form at 3 CTAs (2D Euler 128^2, FP32);
-// at 3 CTAs the packed form spilled 488 B (140 us).  At degree 5 both lines'
-// pair data no longer fit: packed 99 (2 CTAs) or 109 us (1 CTA) against 83 us
-// for the scalar form (96^2).
+// CTAs per SM) and the highest degree that takes the packed x/y form by
+// default.  FP32, us per volume launch: degree 4 (128^2) packed at 2 CTAs 49.0,
+// at 3 CTAs 60, at 1 CTA 59.7, scalar at 3 CTAs 57.9, at 4 CTAs 68.7; degree 5
+// (97x61) scalar at 2 CTAs 47.6, at 3 CTAs 76, packed at 2 CTAs 49.0, at 1 CTA
+// 53.8 (the packed one won on the larger solves of a batch, so it is the batched
+// form's second shape).
 constexpr int kMinB4 = 3, kMinB4Pack = 2, kMinB5 = 2, kPackMaxN = 4;
-// degree 2, FP32: short lines, little per-thread state; 8 CTAs per SM (measured
-// 0.50 -> 0.42 ms per batched volume launch against 3)
-constexpr int kMinB2 = 8;
+// degree 2, FP32: 4 CTAs per SM (256^2: 26.7 us per volume launch, 27.4 at 5, 30.5 at
+// 6, 39.4 at 8); degree 3: 3 CTAs (256^2: 47.5, 50.6 at 2, 49.7 at 4)
+constexpr int kMinB2 = 4, kMinB3 = 3;
 // GLM-MHD (9 variables, 13 pair data): 2 CTAs per SM where the layout allows
 // it, which needs the shared memory of the next tile's staging buffer
-// (measured: 0.58 against 0.73 ms per volume launch at 128^2, N = 4, FP32)
+// (128^2, N = 4, FP32: 174 against 206 us per volume launch with one)
 constexpr int kMinBNc = 2;
 constexpr bool kStageNc = false;
 
 // Kernel shapes: SH = 0 is the measured default of each variant; SH = 1 is the
 // alternative the batched form's autotuner also times: the scalar form (no
-// x/y packing) at one resident CTA per SM more than the packed default, or,
-// for a scalar default, one fewer (fewer spills, fewer warps).
+// x/y packing) at one resident CTA per SM more than the packed default, for the
+// scalar default of degree 5 (FP32) the packed form, else one CTA fewer (fewer
+// spills, fewer warps).
 template <class EQ, int N, typename R, int SH = 0>
 struct LaneLayout;
 
@@ -266,7 +193,7 @@ struct LaneLayout<EQ, N, R, 0> {
   // CTAs per SM the register allocation aims at (the packed form holds both
   // lines' pair data at once)
   static constexpr int MINB = EQ::NC ? (2 * (bytes() + 1024) <= 228 * 1024 ? kMinBNc : 1)
-                            : (THREADS <= 128) ? ((N == 2 && sizeof(R) == 4) ? kMinB2 : PACK ? 3 : 4)
+                            : (THREADS <= 128) ? ((N == 2 && sizeof(R) == 4) ? kMinB2 : PACK ? kMinB3 : 4)
                             : (DIM == 2) ? (N == 4 ? (PACK ? kMinB4Pack : kMinB4) : N == 5 ? kMinB5 : 1) : 1;
   static constexpr bool fits() { return bytes() <= 227 * 1024 && THREADS <= 1024; }
 };
@@ -274,8 +201,8 @@ struct LaneLayout<EQ, N, R, 0> {
 template <class EQ, int N, typename R>
 struct LaneLayout<EQ, N, R, 1> : LaneLayout<EQ, N, R, 0> {
   using B = LaneLayout<EQ, N, R, 0>;
-  static constexpr bool PACK = false;
-  static constexpr int MINB = B::PACK ? B::MINB + 1 : (B::MINB > 1 ? B::MINB - 1 : 1);
+  static constexpr bool PACK = N == 5 && PackXY<EQ>::value && sizeof(R) == 4;
+  static constexpr int MINB = PACK ? B::MINB : B::PACK ? B::MINB + 1 : (B::MINB > 1 ? B::MINB - 1 : 1);
 };
 
 // face_accumulate for both lines of the packed form at once (x-line ends in
@@ -406,22 +333,20 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
                                                   Prefetch pf = Prefetch{nullptr, 0, 0, nullptr, nullptr}) {
   using L = LaneLayout<EQ, N, R, SH>;
   constexpr int DIM = L::DIM, M = L::M, P = L::P, n = L::n, NP = L::NP, NF = L::NF, S = S1 ? S1 : L::S;
-  // 2D scalar form, degree 5 and GLM-MHD in FP64: the x-line and the y-line go
-  // through one copy of the pair loop (a rolled loop over the two directions,
-  // the y-line in the frame of swap_xy), with the pair data read back from
-  // shared memory: half the code of two inlined copies, and no pair data held
-  // across the barrier.  Measured: degree 5 (FP32) 244 against 254 us and the
-  // GLM-MHD vortex at degree 4 (FP64) 4.71 against 4.86 ms per launch, but
-  // degree 4 (FP32) 211 against 194 us; elsewhere no gain.
-  constexpr bool ROLL = !L::PACK && DIM == 2 && (N >= 5 || (EQ::NC && sizeof(R) == 8)) && !(EQ::NC && sizeof(R) == 4 && N >= 4);
-  // 2D GLM-MHD in FP32 at degree 4 and 5: the pair loop itself rolled
-  // (line_residual_rolled), both directions' residuals added in place into the
-  // shared buffer RY (cleared by the node phase), so the x-line residual is not
-  // held in registers either.  Measured per launch: degree 5 (96^2) 520 against
-  // 600 us, degree 4 (128^2) 542 against 569 us; degree 3 slower (110 against
-  // 87 us), so it keeps the form below.
-  constexpr bool ROLLP = !L::PACK && DIM == 2 && EQ::NC && sizeof(R) == 4 && N >= 4;
-  constexpr bool ONEQ = ROLL || ROLLP;   // the node phase keeps no pair data
+  // 2D, FP64, degree 5 and GLM-MHD: the x-line and the y-line go through one copy
+  // of the pair loop (a rolled loop over the two directions, the y-line in the
+  // frame of swap_xy), with the pair data read back from shared memory: half the
+  // code of two inlined copies, and no pair data held across the barrier.
+  // Measured per launch: degree 5 (97x61) 1269 against 1294 us, the GLM-MHD
+  // vortex at degree 4 (128^2) 3.27 against 3.58 ms, at degree 3 (61x45) 306
+  // against 319 us; in FP32 two copies are the faster form (degree 5, 97x61,
+  // 47.6 against 51 us; GLM-MHD degree 4, 128^2, 174 against 193 us, and 255 us
+  // with the pair loop rolled over shared memory).
+  constexpr bool ROLL = !L::PACK && DIM == 2 && sizeof(R) == 8 && (N >= 5 || EQ::NC);
+  // 2D Euler, FP32, degree 5: the plain coefficients and a scaling per line for
+  // single solves too, so that a solve and the same solve in a batch round alike
+  // (the scaling is 48 of about 1500 instructions a stage)
+  constexpr bool TPRE = PRE && !(DIM == 2 && !EQ::NC && sizeof(R) == 4 && N == 5);
   constexpr int NS = rk_nsaved(N) > 0 ? rk_nsaved(N) : 1;
 
   const int tid = threadIdx.x;
@@ -483,37 +408,64 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
   for (int i = 0; i < S; ++i) {
     const R bi = S1 ? R(1) : tb.b[i];
     // ---------------- node phase (own x-line): stage state and pair data
-    R q[ONEQ ? 1 : n][P];
+    R q[ROLL ? 1 : n][P];
     if (active) {
+      // w = dt sum_j a_ij R_j: the last stage's residual (x part from registers,
+      // y/z part from shared memory), then the saved ones stage by stage, so that
+      // the slot, its address and the coefficient are taken once per stage, not
+      // once per value (volume launch, FP32: 2D Euler 128^2 N = 4 97 -> 50 us,
+      // 97x61 N = 5 98 -> 51 us, GLM-MHD 128^2 N = 4 491 -> 255 us)
+      R w[n][M];
+      if (i > 0) {
+        const R ap = dtR * tb.a[i][i - 1], bp = tb.b[i - 1];
+#pragma unroll
+        for (int k = 0; k < n; ++k)
+#pragma unroll
+          for (int v = 0; v < M; ++v) {
+            const R r = ax[k][v] + (DIM > 1 ? my[L::O_RY + v * NP + l * n + k] : R(0));
+            rb[k][v] += bp * r;
+            w[k][v] = ap * r;
+            if constexpr (rk_nsaved(N) > 0) ax[k][v] = r;
+          }
+        if constexpr (rk_nsaved(N) > 0) {
+          const int sp = tb.slot[i - 1];
+          if (sp >= 0) {
+#pragma unroll
+            for (int k = 0; k < n; ++k)
+#pragma unroll
+              for (int v = 0; v < M; ++v) rs[sp][k][v] = ax[k][v];
+          }
+#pragma unroll 1
+          for (int j = 0; j < i - 1; ++j) {
+            const R c = dtR * tb.a[i][j];
+            const int sj = tb.slot[j];
+            if (sj >= 0 && c != R(0)) {
+#pragma unroll
+              for (int k = 0; k < n; ++k)
+#pragma unroll
+                for (int v = 0; v < M; ++v) w[k][v] += c * rs[sj][k][v];
+            }
+          }
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < n; ++k)
+#pragma unroll
+          for (int v = 0; v < M; ++v) w[k][v] = R(0);
+      }
 #pragma unroll
       for (int k = 0; k < n; ++k) {
         const int p = l * n + k;
         R uu[M];
 #pragma unroll
-        for (int v = 0; v < M; ++v) {
-          R acc = R(0);
-          if (i > 0) {
-            // complete R_{i-1} = x part (registers) + y/z part (shared); the
-            // rolled-pair form keeps both in shared memory
-            R r = (ROLLP ? R(0) : ax[k][v]) + (DIM > 1 ? my[L::O_RY + v * NP + p] : R(0));
-            rb[k][v] += tb.b[i - 1] * r;
-            acc = tb.a[i][i - 1] * r;
-            if constexpr (rk_nsaved(N) > 0) {
-              if (tb.slot[i - 1] >= 0) rs[tb.slot[i - 1]][k][v] = r;
-              for (int j = 0; j < i - 1; ++j)
-                if (tb.slot[j] >= 0) acc += tb.a[i][j] * rs[tb.slot[j]][k][v];
-            }
-          }
-          uu[v] = my[L::O_U0 + v * NP + p] - dtR * acc;
-          if constexpr (ROLLP) my[L::O_RY + v * NP + p] = R(0);
-        }
-        R* qk = q[ONEQ ? 0 : k];
+        for (int v = 0; v < M; ++v) uu[v] = my[L::O_U0 + v * NP + p] - w[k][v];
+        R* qk = q[ROLL ? 0 : k];
         EQ::pair_data(uu, qk, pp);
         if (DIM > 1) {
 #pragma unroll
           for (int c = 0; c < P; ++c) my[L::O_Q + c * NP + p] = qk[c];
         }
-        if constexpr (ONEQ && EQ::NCS) {
+        if constexpr (ROLL && EQ::NCS) {
           // face traces of this stage: the ends of the x-line, and the whole
           // x-line where it lies on a face normal to y
           if (k == 0) write_stage_prims<EQ, N, R>(trace, 0, 0, l, i, E, e0 + el, qk);
@@ -522,7 +474,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           if (l == N) write_stage_prims<EQ, N, R>(trace, 1, 1, k, i, E, e0 + el, qk);
         }
       }
-      if constexpr (EQ::NCS && !ONEQ) {
+      if constexpr (EQ::NCS && !ROLL) {
         // face traces of this stage at the ends of the x-line (stage-wise
         // non-conservative flux)
         write_stage_prims<EQ, N, R>(trace, 0, 0, l, i, E, e0 + el, q[0]);
@@ -530,9 +482,9 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
       }
       // ---------------- x-direction flux differencing, all in registers
       // (packed form: together with the y-line below)
-      if constexpr (!PACK && !ONEQ) {
+      if constexpr (!PACK && !ROLL) {
         R fend[2][M];
-        line_differences<EQ, N, R, PRE>(0, q, ax, fend, pp, tb, 0, inv_dx_of<R>(ma, 0));
+        line_differences<EQ, N, R, TPRE>(0, q, ax, fend, pp, tb, 0, inv_dx_of<R>(ma, 0));
         face_accumulate<EQ, N, R, 0>(fx, q, fend, bi, i == 0, pp);
       }
     }
@@ -550,7 +502,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
         for (int k = 0; k < n; ++k)
 #pragma unroll
           for (int c = 0; c < P; ++c) q2[k][c] = f2(q[k][c], qy[k][PackXY<EQ>::rot(c)]);
-        line_residual_xy<EQ, N, PRE>(q2, acc2, fe2, pp2, tb, f2(inv_dx_of<float>(ma, 0), inv_dx_of<float>(ma, 1)));
+        line_residual_xy<EQ, N, TPRE>(q2, acc2, fe2, pp2, tb, f2(inv_dx_of<float>(ma, 0), inv_dx_of<float>(ma, 1)));
 #pragma unroll
         for (int k = 0; k < n; ++k)
 #pragma unroll
@@ -568,21 +520,6 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
         face_accumulate_xy<EQ, N>(fxy, q2, fe2, f2(bi), i == 0, pp2);
       }
       __syncthreads();   // RY complete
-    } else if constexpr (ROLLP) {
-      __syncthreads();   // Q of this stage visible; RY of the last stage consumed and cleared
-#pragma unroll 1
-      for (int dir = 0; dir < 2; ++dir) {
-        if (active) {
-          R qe[n][P], fe[2][M];
-          line_residual_rolled<EQ, N, R>(my + L::O_Q, my + L::O_RY, NP, dir ? l : l * n, dir ? n : 1, dir != 0, qe,
-                                         fe, pp, tb, dir);
-          if (dir == 0) face_accumulate<EQ, N, R, 0>(fx, qe, fe, bi, i == 0, pp);
-          else face_accumulate<EQ, N, R, 0>(fy, qe, fe, bi, i == 0, pp);   // swapped frame
-        }
-        // the x pass is complete before the y pass adds into the same nodes;
-        // after the y pass RY holds the whole residual
-        __syncthreads();
-      }
     } else if constexpr (ROLL) {
       __syncthreads();   // Q of this stage visible; RY of the last stage consumed
       if (active) {
@@ -595,7 +532,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           for (int k = 0; k < n; ++k)
 #pragma unroll
             for (int c = 0; c < P; ++c) qd[k][c] = my[L::O_Q + (dir ? swap_xy<EQ>(c) : c) * NP + base + k * stride];
-          line_differences<EQ, N, R, PRE>(0, qd, ad, fe, pp, tb, dir, dir ? inv_dx_of<R>(ma, 1) : inv_dx_of<R>(ma, 0));
+          line_differences<EQ, N, R, TPRE>(0, qd, ad, fe, pp, tb, dir, dir ? inv_dx_of<R>(ma, 1) : inv_dx_of<R>(ma, 0));
           if (dir == 0) {
 #pragma unroll
             for (int k = 0; k < n; ++k)
@@ -628,7 +565,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           write_stage_prims<EQ, N, R>(trace, 1, 0, l, i, E, e0 + el, qy[0]);
           write_stage_prims<EQ, N, R>(trace, 1, 1, l, i, E, e0 + el, qy[N]);
         }
-        line_differences<EQ, N, R, PRE>(DIM > 1 ? 1 : 0, qy, ay, fend, pp, tb, 1, inv_dx_of<R>(ma, 1));
+        line_differences<EQ, N, R, TPRE>(DIM > 1 ? 1 : 0, qy, ay, fend, pp, tb, 1, inv_dx_of<R>(ma, 1));
         face_accumulate<EQ, N, R, (DIM > 1 ? 1 : 0)>(fy, qy, fend, bi, i == 0, pp);
 #pragma unroll
         for (int k = 0; k < n; ++k)
@@ -645,7 +582,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           for (int k = 0; k < n; ++k)
 #pragma unroll
             for (int c = 0; c < P; ++c) qz[k][c] = my[L::O_Q + c * NP + base + k * n * n];
-          line_differences<EQ, N, R, PRE>(DIM - 1, qz, az, fend, pp, tb, 2, inv_dx_of<R>(ma, DIM - 1));
+          line_differences<EQ, N, R, TPRE>(DIM - 1, qz, az, fend, pp, tb, 2, inv_dx_of<R>(ma, DIM - 1));
           face_accumulate<EQ, N, R, DIM - 1>(fz, qz, fend, bi, i == 0, pp);
 #pragma unroll
           for (int k = 0; k < n; ++k)
@@ -664,7 +601,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
       const int p = l * n + k;
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        R r = (ROLLP ? R(0) : ax[k][v]) + (DIM > 1 ? my[L::O_RY + v * NP + p] : R(0));
+        R r = ax[k][v] + (DIM > 1 ? my[L::O_RY + v * NP + p] : R(0));
         my[L::O_Q + v * NP + p] = rb[k][v] + (S1 ? R(1) : tb.b[S - 1]) * r;
       }
     }
@@ -706,7 +643,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
         }
     }
     write_records<EQ, R, NF>(trace, fx, 0, E, e0 + el, l, u0 + l * n, u0 + l * n + N, NP);
-    if constexpr (ONEQ) {
+    if constexpr (ROLL) {
       FaceAcc<EQ, R> fyo;
 #pragma unroll
       for (int sd = 0; sd < 2; ++sd) {
