@@ -242,6 +242,7 @@ void fill_launch_ctx(const cr_mesh_desc& d, const VariantOps& o, LaunchCtx* plc)
   }
   for (int k = 0; k < 3; ++k) lc.ma.inv_dx_f[k] = (float)lc.ma.inv_dx[k];
   lc.ma.gamma_f = (float)d.gamma;
+  lc.ma.gm1_f = (float)(d.gamma - 1.0);
   lc.ma.c_h_f = (float)d.c_h;
   lc.ma.cfl = d.cfl;
   lc.ma.dt_fixed = d.dt_fixed;

@@ -116,6 +116,7 @@ extern "C" int cr_step_noalloc(const cr_mesh_desc* desc, const double* u_in, dou
   }
   for (int k = 0; k < 3; ++k) lc.ma.inv_dx_f[k] = (float)lc.ma.inv_dx[k];
   lc.ma.gamma_f = (float)d.gamma;
+  lc.ma.gm1_f = (float)(d.gamma - 1.0);
   lc.ma.c_h_f = (float)d.c_h;
   lc.ma.cfl = d.cfl;
   lc.ma.dt_fixed = d.dt_fixed;

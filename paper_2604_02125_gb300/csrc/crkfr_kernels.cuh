@@ -66,7 +66,7 @@ struct MeshArgs {
   double inv_dx[3];
   double cfl, dt_fixed;
   double gamma, c_h;
-  float inv_dx_f[3], gamma_f, c_h_f;   // FP32 copies (no conversions on the FP64 pipe)
+  float inv_dx_f[3], gamma_f, gm1_f, c_h_f;   // FP32 copies (no conversions on the FP64 pipe); gm1 = gamma - 1
   int tma_ok;           // state base 16-byte aligned and E * NP even: whole tiles can be bulk-copied
 };
 template <typename R> __device__ __forceinline__ R inv_dx_of(const MeshArgs& ma, int d);
@@ -576,6 +576,44 @@ __device__ __forceinline__ bool physical_state(const double* uu, const MeshArgs&
     for (int v = 0; v < EQ::M; ++v) uf[v] = d2f_rz(uu[v]);
     if constexpr (EQ::NC) return EQ::physical(uf, ma.gamma_f, ma.c_h_f, lam, ma.inv_dx_f);
     else return EQ::physical(uf, ma.gamma_f, lam, ma.inv_dx_f);
+  }
+}
+
+// A lower bound (FP32, rounded toward zero) of the maximum that the CFL slot
+// will hold: what the warps sharing this warp's word have reduced so far.
+__device__ __forceinline__ float lambda_seen(const DevState* st, int slot) {
+  const unsigned word = (blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) % kLamSpread;
+  const unsigned long long b = *reinterpret_cast<const volatile unsigned long long*>(&st->lam_bits[slot][word]);
+  return d2f_rz(__longlong_as_double((long long)b));
+}
+
+// Physicality and wave speeds of the warp's nodes (on: the lane has one) in the
+// FP64 form.  Only a node that could raise the maximum is evaluated in FP64:
+// one whose FP32 upper bound is below thr, a lower bound of the maximum, and
+// which is certainly physical cannot change the result, which stays exactly the
+// FP64 maximum over all nodes.  The evaluation (a division, square roots, about
+// thirty instructions on the FP64 pipe) was half of this kernel's FP64 work.
+// Called by whole warps; thr is raised to the warp's maximum.
+template <class EQ>
+__device__ __forceinline__ void wave_speeds_fp64(bool on, const double* uu, const MeshArgs& ma, float& thr, double& lam,
+                                                 bool& bad) {
+  bool need = false;
+  if (on) {
+    float uf[EQ::M], up;
+#pragma unroll
+    for (int v = 0; v < EQ::M; ++v) uf[v] = d2f_rz(uu[v]);
+    const bool sure = EQ::speed_bound(uf, MeshSpeeds{ma.gamma_f, ma.gm1_f, ma.c_h_f, ma.inv_dx_f}, up);
+    need = !sure || !(up < thr);
+  }
+  if (__any_sync(0xffffffffu, need)) {
+    if (need) {
+      double lk;
+      bad = !physical_state<EQ, double>(uu, ma, lk) || bad;
+      lam = fmax(lam, lk);
+    }
+    // non-negative floats order like their bits; fmaxf drops the NaN of a value
+    // beyond the FP32 range, and thr stays the bound it was
+    thr = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(fmaxf(thr, d2f_rz(lam)))));
   }
 }
 

@@ -243,6 +243,12 @@ __device__ __forceinline__ float speed_sqrt(float x) {
   return r;
 }
 
+// what the FP32 bound of the wave speeds needs of the mesh
+struct MeshSpeeds {
+  float gamma, gm1, c_h;   // gm1 = gamma - 1
+  const float* inv_dx;
+};
+
 // ---------------------------------------------------------------------------
 // Compressible Euler in DIM dimensions: u = (rho, rho v_1..rho v_DIM, E).
 // Pair data q = (rho, v_1..v_DIM, p, aux); aux = rho/p for the EC flux,
@@ -381,6 +387,28 @@ struct Euler {
   __device__ __forceinline__ static void ncg(int, const R*, R*) {}
   template <typename R>
   __device__ __forceinline__ static void nc_apply(int, const R*, const R*, R*) {}
+
+  // An upper bound of sum_d lambda_d / dx_d from the FP32 truncation of a state;
+  // returns whether the state is certainly physical (else the bound says
+  // nothing).  With e = 2^-23: the inputs, the reciprocal and the roundings leave
+  // |p - p_32| < 16 e (gamma - 1)(E + |m|^2/(2 rho)) and every other factor
+  // within a few e; the bound takes p at its upper end and 32 e on the sum.
+  // Magnitudes whose FP32 parts could underflow are not certain.
+  __device__ __forceinline__ static bool speed_bound(const float* u, const MeshSpeeds& ms, float& up) {
+    const float e16 = 16.0f / 8388608.0f;
+    const float rho = u[0], Et = u[DIM + 1], ir = fast_rcp(rho);
+    float ke = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) ke += u[1 + k] * u[1 + k];
+    const float kr = 0.5f * ke * ir, gm1 = ms.gm1;
+    const float p = gm1 * (Et - kr), dp = e16 * gm1 * (Et + kr);
+    const float c = speed_sqrt(ms.gamma * (p + dp) * ir);
+    float s = 0.0f;
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) s += (fabsf(u[1 + k]) * ir + c) * ms.inv_dx[k];
+    up = s * (1.0f + 2.0f * e16);
+    return rho > 1e-30f && p - dp > 1e-25f && up < 1e38f;
+  }
 
   // physicality of a conserved state (rho > 0, p > 0, finite) and sum_d lambda_d / dx_d
   template <typename T>
@@ -546,6 +574,26 @@ struct GlmMhd {
     out[6] += q[2] * g0;
     out[7] += q[3] * g0;
     out[8] += q[1 + d] * g1;
+  }
+
+  // as Euler's speed_bound; the root's argument takes 32 e of s^2 on top
+  __device__ __forceinline__ static bool speed_bound(const float* u, const MeshSpeeds& ms, float& up) {
+    const float e16 = 16.0f / 8388608.0f;
+    const float rho = u[0], ir = fast_rcp(rho), gm1 = ms.gm1;
+    const float BB = u[5] * u[5] + u[6] * u[6] + u[7] * u[7];
+    const float q = 0.5f * ((u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * ir + BB + u[8] * u[8]);
+    const float p = gm1 * (u[4] - q), dp = e16 * gm1 * (u[4] + q);
+    const float a2 = ms.gamma * (p + dp) * ir, s = (a2 + BB * ir) * (1.0f + e16);
+    float tot = 0.0f;
+#pragma unroll
+    for (int d = 0; d < 2; ++d) {
+      const float bd2 = u[5 + d] * u[5 + d] * ir * (1.0f - e16);
+      const float arg = fmaxf(s * s * (1.0f + 2.0f * e16) - 4.0f * ms.gamma * fmaxf(p - dp, 0.0f) * ir * bd2, 0.0f);
+      const float cf = speed_sqrt(0.5f * (s + speed_sqrt(arg) * (1.0f + e16)));
+      tot += (fabsf(u[1 + d]) * ir + fmaxf(cf, ms.c_h)) * ms.inv_dx[d];
+    }
+    up = tot * (1.0f + 2.0f * e16);
+    return rho > 1e-30f && p - dp > 1e-25f && up < 1e38f;
   }
 
   template <typename T>

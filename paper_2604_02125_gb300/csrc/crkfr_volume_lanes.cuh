@@ -810,76 +810,52 @@ k_volume_lanes_stage(const double* __restrict__ u, R* __restrict__ rbar, R* __re
 namespace crk {
 
 // ---------------------------------------------------------------------------
-// Face + update kernel, lane form: 32 elements per CTA, warp = x-line index,
-// lane = element.  Every face record a warp loads (own and neighbour) is a run
-// of 32 consecutive elements of the [DIM][2][NF][C][E] trace array, and face
-// membership is uniform across the warp.  u^n (FP64) and Rbar are staged
-// through shared memory with coalesced loads; u^{n+1} leaves the same way.
+// Face + update kernel, lane form: 32 elements per CTA.  The jumps are computed
+// with warp = face node, lane = element (every record a warp loads, own and
+// neighbour, is a run of 32 consecutive elements of the [DIM][2][NF][C][E] trace
+// array), the update with a thread per node in memory order.
 // ---------------------------------------------------------------------------
 template <class EQ, int N, typename R>
 struct FaceLaneLayout {
   static constexpr int DIM = EQ::DIM, M = EQ::M, n = N + 1;
   static constexpr int NP = ipow(n, DIM), NF = NP / n;
   static constexpr int THREADS = 32 * NF;
-  // jumps of the faces normal to y (and z): [DIM-1][side][face node][M][32 elements]
-  static constexpr int NJ = (DIM - 1) * 2 * NF;
-  static constexpr size_t bytes() { return sizeof(R) * (size_t)NJ * M * 32; }
+  // scaled jumps of every face: [DIM][side][M][face node][32 elements], rows of
+  // LD values (phase A writes a row per warp; in phase B the lanes of a warp
+  // read several face nodes of few elements: 2 f + e falls into distinct banks)
+  static constexpr int LD = 34;
+  __host__ __device__ static constexpr int jump(int d, int side, int v) { return ((d * 2 + side) * M + v) * NF * LD; }
+  static constexpr size_t bytes() { return sizeof(R) * (size_t)jump(DIM, 0, 0); }
   static constexpr bool fits() { return THREADS <= 1024 && bytes() <= 227 * 1024; }
+  // Register budget of the face kernels, in resident threads per SM: the update
+  // waits for memory, and registers spent on loads ahead of phase A (96 of
+  // them) cost more warps than they hid.  us per launch, FP32, budget none /
+  // 1024 / 1280 / 1536: 2D Euler 256^2 N = 3 29.8 / 23.0 / 21.0 / 22.7, TGV
+  // 64^3 N = 3 797 / 559 / 556 / 513; GLM-MHD 128^2 N = 4 none / 768 / 1024 /
+  // 1536 57.6 / 29.0 / 29.9 / 52 (spills); 64 batched solves 267 / 234 (1024) /
+  // 221 (1152) / 228 (1280); RKFR 256^2 176 / 126 / 126 / 129.
+  static constexpr int minb(int t) { return t / THREADS > 1 ? t / THREADS : 1; }
+  static constexpr int MINB = minb(sizeof(R) == 8 ? 512 : EQ::NC ? 768 : DIM == 3 ? 1536 : 1280), MINB1 = minb(1152);
 };
-
-// n contiguous values starting at src (vector loads where the alignment
-// allows; COH: through L2, for data written earlier in the same launch)
-template <int n, typename T, bool COH = false>
-__device__ __forceinline__ void load_line(const T* __restrict__ src, T (&out)[n]) {
-  if constexpr (sizeof(T) == 4 && n % 4 == 0) {
-#pragma unroll
-    for (int k = 0; k < n / 4; ++k) {
-      const float4 t = ldx<COH>(reinterpret_cast<const float4*>(src) + k);
-      out[4 * k] = t.x; out[4 * k + 1] = t.y; out[4 * k + 2] = t.z; out[4 * k + 3] = t.w;
-    }
-  } else if constexpr (sizeof(T) == 8 && n % 2 == 0) {
-#pragma unroll
-    for (int k = 0; k < n / 2; ++k) {
-      const double2 t = ldx<COH>(reinterpret_cast<const double2*>(src) + k);
-      out[2 * k] = t.x; out[2 * k + 1] = t.y;
-    }
-  } else {
-#pragma unroll
-    for (int k = 0; k < n; ++k) out[k] = ldx<COH>(src + k);
-  }
-}
-template <int n>
-__device__ __forceinline__ void store_line(float* __restrict__ dst, const float (&in)[n]) {
-  if constexpr (n % 4 == 0) {
-#pragma unroll
-    for (int k = 0; k < n / 4; ++k)
-      reinterpret_cast<float4*>(dst)[k] = make_float4(in[4 * k], in[4 * k + 1], in[4 * k + 2], in[4 * k + 3]);
-  } else {
-#pragma unroll
-    for (int k = 0; k < n; ++k) dst[k] = in[k];
-  }
-}
-template <int n>
-__device__ __forceinline__ void store_line(double* __restrict__ dst, const double (&in)[n]) {
-  if constexpr (n % 2 == 0) {
-#pragma unroll
-    for (int k = 0; k < n / 2; ++k) reinterpret_cast<double2*>(dst)[k] = make_double2(in[2 * k], in[2 * k + 1]);
-  } else {
-#pragma unroll
-    for (int k = 0; k < n; ++k) dst[k] = in[k];
-  }
-}
 
 // One tile of 32 elements starting at e0 (sj: the CTA's shared memory; slot:
 // step parity of the CFL reduction).
 //
-// Phase A: every warp computes the Rusanov jumps of 2 DIM face nodes of each
-// of its 32 elements: the two x-face nodes at the ends of its own x-line, and
-// face node f = l of both faces normal to y (and z), whatever x-line they lie
-// on, into shared memory -- the same record loads for every warp.
-// Phase B: each thread forms the increment of its x-line (eq.
-// crkfr.non.cons.final), the CFL reduction runs, and u^{n+1} is stored last,
-// after the reduction's atomics.
+// Phase A (warp = line index l, lane = element): every warp computes the Rusanov
+// jumps of face node f = l of all 2 DIM faces of its 32 elements, scaled by
+// their correction factor, into shared memory: every record load is a run of 32
+// elements, the same loads for every warp.
+// Phase B (thread = node, in memory order): the tile's values of a variable are
+// n contiguous runs of the CTA's threads; each node's increment (eq.
+// crkfr.non.cons.final) is -dt R-bar plus the jumps of the faces it lies on,
+// then the update, the CFL reduction and the store.  u^n, R-bar and u^{n+1} move
+// in whole lines; with a thread per x-line (lane = element) each access of a
+// warp touched 32 different lines, 20 x 32 of them per warp against 72 of the
+// records (2D Euler, N = 3).  us per launch against that form, FP32: 2D Euler
+// 256^2 N = 3 28.4 -> 21.0 (5.8 TB/s of the algorithmic 116 B per node), 128^2 N = 4
+// 18.9 -> 12.8, TGV 64^3 649 -> 513, GLM-MHD 128^2 N = 4 57.4 -> 29.0, RKFR 256^2
+// 151 -> 124, 64 batched solves 329 -> 221; FP64 within 4% either way (its
+// FP64 pipe is the bound).
 // RK = true: stage mode of the multi-stage RKFR step (RkStage): the increment
 // is the stage's K_j, combined with the earlier stages' into the next stage
 // state (eq. rkfr1) or, at the last stage, into u^{n+1} (eq. rkfr2).
@@ -901,139 +877,133 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
                                                 R dt_fused = R(0), const unsigned char* __restrict__ touched = nullptr,
                                                 double* __restrict__ uout = nullptr) {
   using L = FaceLaneLayout<EQ, N, R>;
-  constexpr int DIM = L::DIM, M = L::M, n = L::n, NP = L::NP, NF = L::NF;
+  constexpr int DIM = L::DIM, M = L::M, n = L::n, NP = L::NP, NF = L::NF, T = L::THREADS, LD = L::LD;
   constexpr bool F32 = sizeof(R) == 4;
   const int tid = threadIdx.x;
-  const int l = tid >> 5, el = tid & 31;
   const long long E = ma.E;
   // a volume CTA that timed out left its records unwritten: leave u^n as it is
   if constexpr (!FUSED) {
     if (st->status & ST_TIMEOUT) return;
   }
-  const unsigned e = e0 + el;
-  const bool active = (long long)e0 + el < E && !(touched && touched[e]);
   const R dtR = FUSED ? dt_fused : step_dt<R>(st);
+  const int nel = (int)min(32LL, E - (long long)e0);
+  const size_t vs = (size_t)E * NP;   // values per variable
+  const size_t g0 = (size_t)e0 * NP + tid;
 
-  // own x-line: Rbar and u^n (N+1 contiguous values per variable), loads issued first
-  R rb[M][n];
-  double un[M][n];
-  unsigned ec[3] = {0, 0, 0};
-  R Jm[M], Jp[M];
-  if (active) {
+  // ---- phase A: scaled jumps, -dt J^- g_R'(1)/dx at the xi = 1 faces and
+  // +dt J^+ (-g_L'(0))/dx at the xi = 0 faces
+  {
+    const int l = tid >> 5, el = tid & 31;
+    const unsigned e = e0 + el;
+    if (el < nel && !(touched && touched[e])) {
+      unsigned ec[3] = {0, 0, 0};
+      elem_coords<DIM>(e, ma, ec);
 #pragma unroll
-    for (int v = 0; v < M; ++v) {
-      const size_t g = ((size_t)v * E + e) * NP + l * n;
-      load_line<n, R, FUSED>(rbar + g, rb[v]);
-      load_line<n>(u + g, un[v]);
+      for (int d = 0; d < DIM; ++d)
+#pragma unroll
+        for (int side = 1; side >= 0; --side) {
+          R J[M];
+          face_jump<EQ, N, R, FUSED>(trace, E, d, side, e, neighbour_of(e, ec, d, side ? +1 : -1, ma), l, J, pp, tb);
+          const R sc = side ? -(dtR * tb.iwN * inv_dx_of<R>(ma, d)) : dtR * tb.iw0 * inv_dx_of<R>(ma, d);
+#pragma unroll
+          for (int v = 0; v < M; ++v) sj[L::jump(d, side, v) + l * LD + el] = mulr(sc, J[v]);
+        }
     }
-    elem_coords<DIM>(e, ma, ec);
-    // ---- phase A: x faces at the own line's ends, face node l of the y / z faces
-    face_jump<EQ, N, R, FUSED>(trace, E, 0, 1, e, neighbour_of(e, ec, 0, +1, ma), l, Jm, pp, tb);
-    face_jump<EQ, N, R, FUSED>(trace, E, 0, 0, e, neighbour_of(e, ec, 0, -1, ma), l, Jp, pp, tb);
-#pragma unroll
-    for (int d = 1; d < DIM; ++d)
-#pragma unroll
-      for (int side = 0; side < 2; ++side) {
-        R J[M];
-        face_jump<EQ, N, R, FUSED>(trace, E, d, side, e, neighbour_of(e, ec, d, side ? +1 : -1, ma), l, J, pp, tb);
-        const R sc = side ? -(dtR * tb.iwN * inv_dx_of<R>(ma, d)) : dtR * tb.iw0 * inv_dx_of<R>(ma, d);
-        R* dst = sj + ((size_t)(((d - 1) * 2 + side) * NF + l) * M) * 32 + el;
-#pragma unroll
-        for (int v = 0; v < M; ++v) dst[v * 32] = sc * J[v];
-      }
   }
-  if (DIM > 1) __syncthreads();
+  __syncthreads();
 
-  // ---- phase B: increment of the own x-line, new state, CFL reduction, store
+  // ---- phase B
   R lam = R(0);
   bool bad = false;
-  if (active) {
-    const int cy = DIM >= 2 ? l % n : 0;
-    const int cz = DIM == 3 ? l / n : 0;
-    R du[n][M];
-#pragma unroll
-    for (int k = 0; k < n; ++k)
-#pragma unroll
-      for (int v = 0; v < M; ++v) du[k][v] = mulr(-dtR, rb[v][k]);
-    {
-      // - dt J^- g_R'(1)/dx + dt J^+ (-g_L'(0))/dx at the x faces
-      const R sR = dtR * tb.iwN * inv_dx_of<R>(ma, 0), sL = dtR * tb.iw0 * inv_dx_of<R>(ma, 0);
-#pragma unroll
-      for (int v = 0; v < M; ++v) { du[N][v] = mad(-sR, Jm[v], du[N][v]); du[0][v] = mad(sL, Jp[v], du[0][v]); }
-    }
-    // y / z faces: whole lines on the face (warp-uniform), scaled jumps from phase A
-#pragma unroll
-    for (int d = 1; d < DIM; ++d) {
-      const int cd = d == 1 ? cy : cz;
-      if (cd == 0 || cd == N) {
-        const int side = cd == N ? 1 : 0;
-#pragma unroll
-        for (int k = 0; k < n; ++k) {
-          const int f = d == 1 ? (k + n * cz) : (k + n * cy);
-          const R* src = sj + ((size_t)(((d - 1) * 2 + side) * NF + f) * M) * 32 + el;
-#pragma unroll
-          for (int v = 0; v < M; ++v) du[k][v] += src[v * 32];
-        }
-      }
-    }
-    if constexpr (RK) {
-      // du is this stage's K_j: keep it for the later stages and combine it
-      // with the earlier ones (a_{j+1,q}, or b_q at the last stage)
-      const bool last = rk.j == rk.s - 1;
-      const size_t nodes = (size_t)E * NP;
+  double* dst = uout ? uout : u;
+  const bool last = !RK || rk.j == rk.s - 1;   // uniform over the grid
+  if (RK && !last) dst = rk.uout;
+  // FP64: a lower bound of the new state's maximum wave speed, from the warps
+  // that have reduced theirs so far
+  float thr = 0.0f;
+  if constexpr (!F32) {
+    if (last) thr = lambda_seen(st, FUSED ? slot : slot ^ 1);
+  }
+#pragma unroll 1
+  for (int j = 0; j < n; ++j) {
+    const int r = tid + j * T, ee = r / NP, p = r % NP;
+    const bool on = ee < nel && !(touched && touched[e0 + ee]);
+    const size_t g = g0 + j * T;
+    double un[M];
+    if (on) {
+      R du[M];
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        const size_t g = ((size_t)v * E + e) * NP + l * n;
-        R kj[n], acc[n];
-        const R cj = last ? tb.b[rk.j] : tb.a[rk.j + 1][rk.j];
+        un[v] = u[g + v * vs];
+        du[v] = ldx<FUSED>(rbar + g + v * vs);
+      }
+      // the jumps of the faces the node lies on (one at most per direction: one
+      // addition, whichever side), then -dt R-bar
+      R t[M];
+      int rem = p;
 #pragma unroll
-        for (int k = 0; k < n; ++k) { kj[k] = du[k][v]; acc[k] = cj * kj[k]; }
-        if (!last) store_line<n>(rk.k + (size_t)rk.j * M * nodes + g, kj);
+      for (int d = 0; d < DIM; ++d) {
+        const int c = rem % n, stride = ipow(n, d);
+        rem /= n;
+        const int f = (p % stride) + (p / (stride * n)) * stride;
+        R td[M];
+#pragma unroll
+        for (int v = 0; v < M; ++v) td[v] = R(0);
+        if (c == 0 || c == N) {
+          const R* src = sj + (c == N ? L::jump(0, 1, 0) : 0) + f * LD + ee;
+#pragma unroll
+          for (int v = 0; v < M; ++v) td[v] = src[L::jump(d, 0, v)];
+        }
+#pragma unroll
+        for (int v = 0; v < M; ++v) t[v] = d == 0 ? td[v] : t[v] + td[v];
+      }
+#pragma unroll
+      for (int v = 0; v < M; ++v) du[v] = mad(-dtR, du[v], t[v]);
+      if constexpr (RK) {
+        // du is this stage's K_j: keep it for the later stages and combine it
+        // with the earlier ones (a_{j+1,q}, or b_q at the last stage)
+        const R cj = last ? tb.b[rk.j] : tb.a[rk.j + 1][rk.j];
+        R acc[M];
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          if (!last) rk.k[(size_t)rk.j * M * vs + v * vs + g] = du[v];
+          acc[v] = mulr(cj, du[v]);
+        }
 #pragma unroll 1
         for (int q = 0; q < rk.j; ++q) {
           const R c = last ? tb.b[q] : tb.a[rk.j + 1][q];
           if (c != R(0)) {
-            R kq[n];
-            load_line<n>(rk.k + (size_t)q * M * nodes + g, kq);
 #pragma unroll
-            for (int k = 0; k < n; ++k) acc[k] += c * kq[k];
+            for (int v = 0; v < M; ++v) acc[v] = mad(c, rk.k[(size_t)q * M * vs + v * vs + g], acc[v]);
           }
         }
 #pragma unroll
-        for (int k = 0; k < n; ++k) du[k][v] = acc[k];
+        for (int v = 0; v < M; ++v) du[v] = acc[v];
       }
-    }
-    // u^{n+1} = u^n + du in FP64
-#pragma unroll
-    for (int k = 0; k < n; ++k) {
-      double uu[M];
+      // u^{n+1} = u^n + du in FP64
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        if constexpr (F32) uu[v] = un[v][k] + f2d_int(du[k][v]);
-        else uu[v] = un[v][k] + du[k][v];
-        un[v][k] = uu[v];
-      }
-      if (!RK || rk.j == rk.s - 1) {
-        R lk;
-        bad = bad || !physical_state<EQ, R>(uu, ma, lk);
-        lam = fmax(lam, lk);
+        if constexpr (F32) un[v] += f2d_int(du[v]);
+        else un[v] += du[v];
+        dst[g + v * vs] = un[v];
       }
     }
+    if constexpr (F32) {
+      if (last && on) {
+        R lk;
+        bad = bad || !physical_state<EQ, R>(un, ma, lk);
+        lam = fmax(lam, lk);
+      }
+    } else {
+      if (last) wave_speeds_fp64<EQ>(on, un, ma, thr, lam, bad);
+    }
   }
-  // the CFL reduction of the new state (RKFR: after the last stage only; the
-  // stage index is uniform over the grid); intermediate stage states go to
-  // rk.uout
-  double* dst = uout ? uout : u;
-  if (RK && rk.j != rk.s - 1) dst = rk.uout;
-  else reduce_lambda<R>(lam, bad, st, FUSED ? slot : slot ^ 1);
-  if (active) {
-#pragma unroll
-    for (int v = 0; v < M; ++v) store_line<n>(dst + ((size_t)v * E + e) * NP + l * n, un[v]);
-  }
+  // the CFL reduction of the new state (RKFR: after the last stage only)
+  if (last) reduce_lambda<R>(lam, bad, st, FUSED ? slot : slot ^ 1);
 }
 
 template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS)
+__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB)
 k_face_update_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
                     DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                     int slot) {
@@ -1044,7 +1014,7 @@ k_face_update_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R*
 // the limited step's elements that the limiter does not touch: the plain
 // update from u^n (uin) into uout (touched: the flags of k_alpha_smooth)
 template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS)
+__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB1)
 k_face_update_lanes_clean(double* __restrict__ uin, double* __restrict__ uout, const R* __restrict__ rbar,
                           const R* __restrict__ trace, const unsigned char* __restrict__ touched,
                           DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
@@ -1056,7 +1026,7 @@ k_face_update_lanes_clean(double* __restrict__ uin, double* __restrict__ uout, c
 
 // face / update part of stage rk.j of the multi-stage RKFR step
 template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS)
+__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB1)
 k_face_stage_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
                    DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                    int slot, const RkStage<R> rk) {
@@ -1143,7 +1113,7 @@ k_volume_batched(const BatchSolve* __restrict__ solves, const BatchTile* __restr
 }
 
 template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS)
+__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB1)
 k_face_batched(const BatchSolve* __restrict__ solves, const BatchTile* __restrict__ tiles, unsigned ntiles,
                const PhysParams<R> pp, const RefTab<R> tb, int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1152,7 +1122,7 @@ k_face_batched(const BatchSolve* __restrict__ solves, const BatchTile* __restric
     const MeshArgs ma = solves[t.solve].ma;
     face_lanes_tile<EQ, N, R>(solves[t.solve].u, (const R*)solves[t.solve].rbar, (const R*)solves[t.solve].trace,
                               solves[t.solve].st, ma, pp, tb, t.e0, slot, reinterpret_cast<R*>(smem_raw));
-    if (EQ::DIM > 1) __syncthreads();   // the jump buffer is reused by the next tile
+    __syncthreads();   // the jump buffer is reused by the next tile
   }
 }
 
