@@ -46,9 +46,9 @@ __device__ __forceinline__ float mulr(float a, float b) { return __fmul_rn(a, b)
 //   L = (a+b) / (2 F(u)),  F(u) = artanh(sqrt u) / sqrt u = 1 + u/3 + u^2/5 + ...
 //   and 1/F(u) = 1 - u/3 - 4u^2/45 - ...
 // FP64: degree 8 below u = 1/16 (least-maximum fits on [0, 1/16], computed with
-// 50 digits; error below 9e-18), inside it degree 3 below u = 2^-13 (error
-// below 2e-19); above 1/16 the ratio a/b exceeds 1.66 and log(a/b) is well
-// conditioned (at u = 1e-4 the quotient's rounding costs log(a/b) 1e-16 / 0.02).
+// 50 digits; error below 9e-18), inside it the series in two FP32 parts below
+// u = 2^-11 (unit_plus); above 1/16 the ratio a/b exceeds 1.66 and log(a/b) is
+// well conditioned (at u = 1e-4 the quotient's rounding costs log(a/b) 1e-16 / 0.02).
 // FP32: degree 3 below u = 0.05 (least-maximum fits on [0, 0.05]; error below
 // 6.2e-9, a tenth of an FP32 ulp of F ~ 1); above it the ratio a/b exceeds 1.57.
 // ---------------------------------------------------------------------------
@@ -59,13 +59,6 @@ __device__ __forceinline__ double series_F(double u) {
 __device__ __forceinline__ double series_invF(double u) {
   return 1.0 + u * (-0.33333333333332982 + u * (-0.088888888890384454 + u * (-0.046560846315972715 + u * (-0.030194023571221005
       + u * (-0.021795885119032539 + u * (-0.016812176252078610 + u * (-0.013121851935549912 + u * -0.014306111787604733)))))));
-}
-// u < 2^-13
-__device__ __forceinline__ double series_F_near(double u) {
-  return 1.0 + u * (0.33333333333338387 + u * (0.19999999793002216 + u * 0.14288427331899907));
-}
-__device__ __forceinline__ double series_invF_near4(double u) {   // 1/(4 F(u))
-  return 0.25 + u * (-0.25 * 0.33333333333334706 + u * (-0.25 * 0.088888888326392527 + u * (-0.25 * 0.046568219037031879)));
 }
 __device__ __forceinline__ float series_F(float u) {
   return 1.0f + u * (0.33333710f + u * (0.19962572f + u * 0.15462606f));
@@ -148,42 +141,95 @@ __device__ __forceinline__ void logmean_pair(float a1, float b1, float a2, float
   }
 }
 
-// the wide polynomials of both means, out of line (twenty instructions on the
-// FP64 pipe that most pairs of a resolved flow do not need)
-static __device__ __noinline__ void series_pair_wide(double u1, double u2, double& g1, double& f2) {
-  g1 = 0.25 * series_invF(u1);
-  f2 = series_F(u2);
+// u = (d/s)^2 as the sum of two FP32 values (relative error about 2^-45), from the
+// bits of d and s: both are scaled by the power of two that takes s to [1, 2).
+// False where that fails: s not a normal number, or |d| >= 2 |s| (or not finite).
+__device__ __forceinline__ bool ratio_squared(double d, double s, float& uh, float& ul) {
+  const unsigned sH = (unsigned)__double2hiint(s), sL = (unsigned)__double2loint(s);
+  const unsigned dH = (unsigned)__double2hiint(d), dL = (unsigned)__double2loint(d);
+  const int es = (int)((sH >> 20) & 0x7FFu), k = (int)((dH >> 20) & 0x7FFu) - es;
+  const float two46 = 1.4210854715202004e-14f;   // 2^-46
+  // leading 24 bits, and the next 23 as a number (2^23 + bits, minus 2^23)
+  const float sh = __uint_as_float(0x3F800000u | (__funnelshift_l(sL, sH, 3) & 0x7FFFFFu));
+  const float sl = (__uint_as_float(0x4B000000u | ((sL >> 6) & 0x7FFFFFu)) - 8388608.0f) * two46;
+  const float sc = __uint_as_float(k > -126 ? (unsigned)(127 + k) << 23 : 0u);
+  const float dh = __uint_as_float(0x3F800000u | (__funnelshift_l(dL, dH, 3) & 0x7FFFFFu)) * sc;
+  const float dl = (__uint_as_float(0x4B000000u | ((dL >> 6) & 0x7FFFFFu)) - 8388608.0f) * (two46 * sc);
+  // quotient by the approximate reciprocal, its remainder divided twice
+  const float r = fast_rcp(sh), q0 = dh * r;
+  const float rem = __fmaf_rn(-q0, sh, dh) + __fmaf_rn(-q0, sl, dl);
+  float q1 = rem * r;
+  q1 = __fmaf_rn(__fmaf_rn(-q1, sh, rem), r, q1);
+  uh = __fmul_rn(q0, q0);
+  ul = __fmaf_rn(q0 + q0, q1, __fmaf_rn(q0, q0, -uh));
+  return (unsigned)(es - 1) < 2046u && k <= 0;
 }
 
-// FP64: the branch compares the high words (u >= 0, and a NaN's is above every
-// bound), which keeps the comparisons off the narrow FP64 pipe that bounds
-// these kernels.  A flow resolved by its mesh mixes pairs below 2^-13 (two
-// thirds of them on the 256^2, N = 3 shear layer) with pairs up to 1e-2; sending
-// the latter to two logarithms (about 150 FP64 instructions with their
-// divisions) instead of the wide polynomials, as a single bound of 1e-4 did,
-// took 124 against 71 us per volume launch on the 64-element 1D wave and 2138
-// against 1846 us on the shear layer (with the three-FMA reciprocal).
+// 1 + u (c1 + u (c2 + u (c3 + u (c4 + u c5)))) for 0 <= u < 2^-11 as a double,
+// times the power of two whose high word is `unit`: the series beyond 1 in two
+// FP32 parts (c1 and c2 too), whose sum is at most 2^-12.6 and right to 2^-57, then
+// added to the bits of the unit as a fixed-point number -- in steps of 2^-52 above
+// 1, of 2^-53 below (NEG: c1 < 0).  Rounding to integers by adding 1.5 2^23.
+template <bool NEG>
+__device__ __forceinline__ double unit_plus(float uh, float ul, float c1h, float c1l, float c2h, float c2l, float c3,
+                                            float c4, float c5, unsigned unit) {
+  const float t = uh * __fmaf_rn(uh, __fmaf_rn(uh, c5, c4), c3);
+  const float mh = __fadd_rn(c2h, t), ml = __fadd_rn(t, -__fadd_rn(mh, -c2h)) + c2l;
+  const float nh = __fmul_rn(uh, mh), nl = __fmaf_rn(uh, mh, -nh) + __fmaf_rn(uh, ml, ul * mh);
+  const float oh = __fadd_rn(c1h, nh), ol = __fadd_rn(nh, -__fadd_rn(oh, -c1h)) + c1l + nl;
+  const float ch = __fmul_rn(uh, oh), cl = __fmaf_rn(uh, oh, -ch) + __fmaf_rn(uh, ol, ul * oh);
+  const float magic = 12582912.0f;   // 1.5 2^23
+  const float x = __fmaf_rn(ch, 2147483648.0f, magic);                       // ch in steps of 2^-31
+  const float rem = __fmaf_rn(-__fadd_rn(x, -magic), 4.656612873077393e-10f, ch) + cl;
+  const float y = __fmaf_rn(rem, NEG ? 9007199254740992.0f : 4503599627370496.0f, magic);
+  const int ih = __float_as_int(x) - 0x4B400000, il = __float_as_int(y) - 0x4B400000;
+  const long long i = (long long)ih * (1ll << (NEG ? 22 : 21)) + il + ((long long)unit << 32);
+  return __longlong_as_double(i);
+}
+
+// the pairs beyond the two-part series: out of line, since most pairs of a
+// resolved flow do not come here
+static __device__ __noinline__ void logmean_pair_far(double a1, double b1, double a2, double b2, double rs2, double& H1,
+                                                     double& T2) {
+  const double s1 = a1 + b1;
+  const double f1 = (a1 - b1) * fast_rcp(s1), f2 = (a2 - b2) * rs2;
+  const double u1 = f1 * f1, u2 = f2 * f2;
+  if (fmax(u1, u2) < LogMeanEps<double>::v) {
+    H1 = s1 * (0.25 * series_invF(u1));
+    T2 = series_F(u2) * rs2;
+  } else {
+    logmean_pair_general(a1, b1, a2, b2, H1, T2);
+  }
+}
+
+// FP64.  The FP64 pipe bounds these kernels (a warp instruction occupies it for
+// about 18 cycles, in which the SM can issue 70 others), so everything that is
+// needed to less than 53 bits is done beside it: the two polynomials' part beyond
+// 1 is a correction below 2^-12.6, two FP32 parts give it to 2^-57, and integer
+// arithmetic adds it to 1.  Nine FP64 instructions a pair (four sums, a
+// three-FMA reciprocal, two products) against 22 with the polynomials in FP64;
+// the result's error is that of its roundings, as there (against 128 bits, for
+// u < 2^-11: 1/F within 9.9e-17 and F within 1.5e-16, root mean square 3.3e-17 and
+// 6.4e-17; FP64 Horner 3.2e-17 and 6.4e-17).  Volume launch: 256^2, N = 3 1558 -> 1227
+// us, 97x61 N = 5 1266 -> 951, 64-element 1D wave 64 -> 53, GLM-MHD 128^2 N = 4 3267 ->
+// 2933.  Above 2^-11 (a/b > 1.045) the degree-8
+// polynomials in FP64, above 1/16 the logarithms (a single FP64 series bound at
+// 1e-4 with logarithms beyond cost 124 against 71 us per volume launch on the
+// 64-element 1D wave and 2138 against 1846 us on the 256^2, N = 3 shear layer).
 __device__ __forceinline__ void logmean_pair(double a1, double b1, double a2, double b2, double& H1, double& T2,
                                              double& rs2) {
   const double s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
-  const double r = fast_rcp(s1 * s2);
-  const double rs1 = s2 * r;
-  rs2 = s1 * r;
-  const double f1 = d1 * rs1, f2 = d2 * rs2;
-  const double u1 = f1 * f1, u2 = f2 * f2;
-  const unsigned h = max((unsigned)__double2hiint(u1), (unsigned)__double2hiint(u2));
-  if (h < 0x3FB00000u) {   // 1/16
-    double g, f;
-    if (h < 0x3F200000u) {   // 2^-13
-      g = series_invF_near4(u1);
-      f = series_F_near(u2);
-    } else {
-      series_pair_wide(u1, u2, g, f);
-    }
-    H1 = s1 * g;
-    T2 = f * rs2;
+  rs2 = fast_rcp(s2);
+  float h1, l1, h2, l2;
+  const bool ok1 = ratio_squared(d1, s1, h1, l1), ok2 = ratio_squared(d2, s2, h2, l2);
+  if (ok1 && ok2 && fmaxf(h1, h2) < 4.8828125e-4f) {   // 2^-11
+    // 1/F = 1 - u/3 - 4u^2/45 - 44u^3/945 - 428u^4/14175 - 10196u^5/467775, F = 1 + u/3 + u^2/5 + ...
+    H1 = s1 * unit_plus<true>(h1, l1, -0.33333334f, 9.9341078e-9f, -0.088888891f, 2.1523899e-9f, -44.0f / 945.0f,
+                              -428.0f / 14175.0f, -10196.0f / 467775.0f, 0x3FD00000u);
+    T2 = rs2 * unit_plus<false>(h2, l2, 0.33333334f, -9.9341078e-9f, 0.2f, -2.9802323e-9f, 1.0f / 7.0f, 1.0f / 9.0f,
+                                1.0f / 11.0f, 0x3FF00000u);
   } else {
-    logmean_pair_general(a1, b1, a2, b2, H1, T2);
+    logmean_pair_far(a1, b1, a2, b2, rs2, H1, T2);
   }
 }
 

@@ -23,10 +23,23 @@ EDGES = [0.0, 1e-12, 2.0 ** -13 * (1 - 1e-9), 2.0 ** -13 * (1 + 1e-9), 1e-3, 0.0
          0.0625 * (1 - 1e-9), 0.0625 * (1 + 1e-9), 0.3]
 
 
+# the FP64 form's two-part series: on both sides of its bound, across the
+# exponents its fixed-point sum spans, and where the corrections vanish
+SERIES_EDGES = [2.0 ** -11 * (1 - 1e-9), 2.0 ** -11 * (1 + 1e-9), 2.0 ** -12, 3e-5, 1e-7, 1e-16, 1e-24, 1e-31]
+
+
+@pytest.mark.parametrize("eq,N", [("euler", 3), ("glm_mhd", 3)])
+@pytest.mark.parametrize("scale", [1.0, 1e-60, 1e60])
+@pytest.mark.parametrize("u", SERIES_EDGES)
+def test_two_part_series(u, scale, eq, N):
+    """scale: density and pressure (and the magnetic energy) far outside the FP32 range."""
+    test_log_mean_branches(u, eq, N, "fp64", 1e-11, scale)
+
+
 @pytest.mark.parametrize("prec,tol", [("fp64", 1e-11), ("fp32", 1e-4)])
 @pytest.mark.parametrize("eq,N", [("euler", 3), ("euler", 4), ("glm_mhd", 3)])
 @pytest.mark.parametrize("u", EDGES)
-def test_log_mean_branches(u, eq, N, prec, tol):
+def test_log_mean_branches(u, eq, N, prec, tol, scale=1.0):
     oracle.build()
     dim = 2
     mesh = inputs.mesh_dict(eq, dim, N, [5, 3], [0.0, 0.0], [1.0, 0.7], 1.4, c_h=0.0 if eq == "euler" else 2.0)
@@ -34,14 +47,15 @@ def test_log_mean_branches(u, eq, N, prec, tol):
     f = np.sqrt(u)
     p = np.arange(n * n)
     odd = ((p % n + p // n) % 2)[None, :]
-    rho = np.where(odd == 1, (1 + f) / (1 - f), 1.0) * np.ones((15, 1))
-    pr = np.where(np.arange(15)[:, None] % 2 == 0, 1.0, rho)
+    rho = scale * np.where(odd == 1, (1 + f) / (1 - f), 1.0) * np.ones((15, 1))
+    pr = np.where(np.arange(15)[:, None] % 2 == 0, scale, rho)
+    root = np.sqrt(scale)
     v = [0.3 + 0.05 * odd * np.ones_like(rho), -0.2 * np.ones_like(rho)]
     if eq == "euler":
         U = inputs.euler_cons(1.4, rho, v, pr)
     else:
         one = np.ones_like(rho)
-        U = inputs.mhd_cons(1.4, rho, v + [0.1 * one], pr, [0.4 * one, 0.3 * one, 0.2 * one], 0.1 * one)
+        U = inputs.mhd_cons(1.4, rho, v + [0.1 * one], pr, [0.4 * root * one, 0.3 * root * one, 0.2 * root * one], 0.1 * root * one)
     s = crkfr.Solver(mesh, prec=prec)
     s.set_state(U)
     s.step(1)
