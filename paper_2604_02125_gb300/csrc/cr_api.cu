@@ -229,7 +229,7 @@ void fill_lim_tab(int N, double alpha_max, LimTab* lt) {
   lt->e_hi_f = (float)(lt->tau * (1.0 + std::log(0.999 / 0.001) / lt->sharp));
 }
 
-void fill_launch_ctx(const cr_mesh_desc& d, const VariantOps& o, LaunchCtx* plc) {
+void fill_launch_ctx(const cr_mesh_desc& d, LaunchCtx* plc) {
   LaunchCtx& lc = *plc;
   std::memset(&lc, 0, sizeof(lc));
   long long E = 1;
@@ -251,7 +251,6 @@ void fill_launch_ctx(const cr_mesh_desc& d, const VariantOps& o, LaunchCtx* plc)
   lc.pp64 = make_phys<double>(d.gamma, d.c_h);
   lc.pp32 = make_phys<float>(d.gamma, d.c_h);
   fill_ref_tables(d.degree_N, d.eq, lc.ma, &lc.tb64, &lc.tb32);
-  lc.epb = default_epb(o);
   int dev = 0;
   cudaGetDevice(&dev);
   lc.sms = 1;
@@ -261,17 +260,6 @@ void fill_launch_ctx(const cr_mesh_desc& d, const VariantOps& o, LaunchCtx* plc)
 // whole 32-element tiles of the state can be fetched with 16-byte bulk copies
 int tma_ok_for(const double* u, long long E, int NP) {
   return ((reinterpret_cast<size_t>(u) & 15) == 0 && ((E * NP) % 2) == 0) ? 1 : 0;
-}
-
-int default_epb(const VariantOps& o) {
-  int epb = 256 / o.NF;
-  if (epb < 1) epb = 1;
-  const size_t cap = 160 * 1024;
-  while (epb > 1 && (size_t)epb * o.vol_bytes_per_elem > cap) --epb;
-  // prefer a whole number of warps
-  for (int e = epb; e >= 1; --e)
-    if ((e * o.NF) % 32 == 0) return e;
-  return epb;
 }
 
 }  // namespace crk
@@ -549,7 +537,7 @@ static int init_single(cr_ctx* c, void* workspace = nullptr) {
   const VariantOps& o = c->ops;
   const long long E = c->E;
   LaunchCtx& lc = c->lc;
-  fill_launch_ctx(d, o, &lc);
+  fill_launch_ctx(d, &lc);
   if (c->limited) fill_lim_tab(d.degree_N, d.alpha_max, &lc.lt);
   c->borrowed = workspace != nullptr;
   size_t off = 0;
@@ -565,7 +553,7 @@ static int init_single(cr_ctx* c, void* workspace = nullptr) {
   lc.u = c->ubuf[0];
   if (rc != CR_OK) { free_single(c); return rc; }
   lc.ma.tma_ok = tma_ok_for(lc.u, E, o.NP);
-  cudaError_t e = o.set_smem(o.vol_smem(lc.epb));
+  cudaError_t e = o.set_smem();
   if (e != cudaSuccess) { free_single(c); return cuda_status(e); }
   e = cudaMemsetAsync(lc.st, 0, sizeof(DevState), c->stream);
   if (e == cudaSuccess && c->limited) e = cudaMemsetAsync(lc.alpha, 0, sizeof(double) * (size_t)E, c->stream);
@@ -886,9 +874,7 @@ int cr_tuning_info(cr_ctx* c, char* buf, size_t len) {
                   "{\"scheme\": \"%s\", \"step\": \"%s\", \"volume\": \"%s\", \"elements_per_cta\": %d, "
                   "\"face\": \"%s\"}",
                   c->desc[0].scheme == CR_SCHEME_RKFR ? "rkfr" : "crkfr", c->fused ? "fused" : "split",
-                  c->ops.lanes ? "lanes" : "tile",
-                  c->ops.lanes ? 32 : c->lc.epb,
-                  c->limited ? "limited per-node" : (c->ops.threads_face > 0 ? "lanes" : "per-node"));
+                  "lanes", c->ops.lane_elems, c->limited ? "limited per-node" : "lanes");
     info = tmp;
   }
   std::snprintf(buf, len, "%s", info.c_str());

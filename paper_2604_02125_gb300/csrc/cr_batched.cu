@@ -123,7 +123,7 @@ int batched_init(BatchedCtx** out, const cr_mesh_desc* desc, int n, cudaStream_t
       return CR_EINVAL;
     }
     const VariantOps& o = b->ops[k];
-    fill_launch_ctx(d, o, &b->lc[k]);
+    fill_launch_ctx(d, &b->lc[k]);
     const long long E = b->lc[k].ma.E, nodes = E * o.NP;
     b->nvals[k] = (size_t)o.M * nodes;
     b->off_u[k] = b->total_u;
@@ -161,7 +161,7 @@ int batched_init(BatchedCtx** out, const cr_mesh_desc* desc, int n, cudaStream_t
     hs[k].trace = lc.trace;
     hs[k].st = lc.st;
     hs[k].ntiles = (unsigned)((lc.ma.E + 31) / 32);
-    cudaError_t e = b->ops[k].set_smem(b->ops[k].vol_smem(lc.epb));
+    cudaError_t e = b->ops[k].set_smem();
     if (e != cudaSuccess) { free_all(b); delete b; return st_of(e); }
   }
   // work lists per degree: tiles of all solves of that degree, largest solves first

@@ -21,7 +21,6 @@ struct LaunchCtx {
   PhysParams<float> pp32;
   RefTab<double> tb64;
   RefTab<float> tb32;
-  int epb;            // elements per CTA of the volume kernel (tile form)
   int sms;            // multiprocessors of the device (persistent grids)
   int slot;           // step parity: CFL-reduction slot of the state the next step starts from
   // multi-stage RKFR scratch: stage state u^(j) (FP64, like u) and the
@@ -58,9 +57,7 @@ struct BatchLaunch {
 struct VariantOps {
   int M, NP, NF, C, dim;       // C: components of a face record
   size_t ncs_per_elem;         // stage-wise non-conservative flux: stage-trace values per element after the records
-  size_t vol_bytes_per_elem;   // shared memory per element of the tile volume kernel
-  bool lanes;                  // the lane-form volume kernel is used (32 elements per CTA)
-  size_t (*vol_smem)(int epb); // dynamic shared memory of one volume CTA
+  int lane_elems;              // elements per CTA of the volume kernel
   size_t real_bytes;           // sizeof(R)
   cudaError_t (*volume)(const LaunchCtx&, cudaStream_t);
   cudaError_t (*face_update)(const LaunchCtx&, cudaStream_t);
@@ -82,7 +79,7 @@ struct VariantOps {
   cudaError_t (*step_fused)(const LaunchCtx&, cudaStream_t, int phase);
   cudaError_t (*lambda)(const LaunchCtx&, cudaStream_t);
   cudaError_t (*totals)(const LaunchCtx&, cudaStream_t);
-  cudaError_t (*set_smem)(size_t bytes);
+  cudaError_t (*set_smem)();
   // batched persistent kernels (2D Euler only; null elsewhere)
   cudaError_t (*vol_batched)(const BatchLaunch&, cudaStream_t);
   cudaError_t (*face_batched)(const BatchLaunch&, cudaStream_t);
@@ -134,11 +131,8 @@ bool get_ops(int eq, int dim, int prec, int vol, int N, VariantOps* o, int ncflu
 // subcell widths, logistic threshold and sharpness)
 void fill_lim_tab(int N, double alpha_max, LimTab* lt);
 
-// elements per CTA of the volume kernel used by every context of a variant
-int default_epb(const VariantOps& o);
-
 // mesh arguments, physics parameters and tables of one descriptor (no allocation)
-void fill_launch_ctx(const cr_mesh_desc& d, const VariantOps& o, LaunchCtx* lc);
+void fill_launch_ctx(const cr_mesh_desc& d, LaunchCtx* lc);
 
 // 1 if whole tiles of a state at u (E elements of NP nodes) can be bulk-copied
 int tma_ok_for(const double* u, long long E, int NP);

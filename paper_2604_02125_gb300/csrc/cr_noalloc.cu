@@ -125,12 +125,11 @@ extern "C" int cr_step_noalloc(const cr_mesh_desc* desc, const double* u_in, dou
   lc.pp64 = make_phys<double>(d.gamma, d.c_h);
   lc.pp32 = make_phys<float>(d.gamma, d.c_h);
   fill_ref_tables(d.degree_N, d.eq, lc.ma, &lc.tb64, &lc.tb32);
-  lc.epb = default_epb(o);
   lc.sms = 1;
   if ((e = cudaDeviceGetAttribute(&lc.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return to_status(e);
   lc.ma.tma_ok = tma_ok_for(u_out, E, o.NP);
 
-  if ((e = o.set_smem(o.vol_smem(lc.epb))) != cudaSuccess) return to_status(e);
+  if ((e = o.set_smem()) != cudaSuccess) return to_status(e);
   if (u_out != u_in &&
       (e = cudaMemcpyAsync(u_out, u_in, sizeof(double) * (size_t)o.M * nodes, cudaMemcpyDeviceToDevice, s)) !=
           cudaSuccess)

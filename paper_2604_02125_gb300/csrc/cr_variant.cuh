@@ -29,98 +29,61 @@ template <> struct PPB<float> {
 
 template <class EQ, int N, typename R>
 struct Variant {
-  using L = VolLayout<EQ, N, R>;
   using LL = LaneLayout<EQ, N, R>;
   using PL = PersistLayout<EQ, N, R>;
-  static constexpr bool kLanes = PL::fits();
-  static size_t vol_smem(int epb) { return kLanes ? PL::bytes() : (size_t)epb * L::bytes_per_elem(); }
+  using FL = FaceLaneLayout<EQ, N, R>;
+  static_assert(PL::fits() && FL::fits(), "the lane layouts hold every variant");
   // resident CTAs per SM of the persistent volume kernel (computed once)
   static int vol_occupancy() {
     static int occ = -1;
     if (occ < 0) {
       int nb = 0;
-      if constexpr (kLanes) {
-        cudaFuncSetAttribute(k_volume_lanes<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::bytes());
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes<EQ, N, R>, LL::THREADS, PL::bytes());
-      }
+      cudaFuncSetAttribute(k_volume_lanes<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::bytes());
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes<EQ, N, R>, LL::THREADS, PL::bytes());
       occ = nb > 0 ? nb : 1;
     }
     return occ;
   }
   static cudaError_t volume(const LaunchCtx& c, cudaStream_t s) {
-    if constexpr (kLanes) {
-      const long long ntiles = (c.ma.E + 31) / 32;
-      const long long grid = std::min(ntiles, (long long)c.sms * vol_occupancy());
-      k_volume_lanes<EQ, N, R><<<(unsigned)grid, LL::THREADS, PL::bytes(), s>>>(
-          c.u, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
-    } else {
-      const long long grid = (c.ma.E + c.epb - 1) / c.epb;
-      const int threads = c.epb * L::NF;
-      const size_t smem = (size_t)c.epb * L::bytes_per_elem();
-      k_volume_tile<EQ, N, R><<<(unsigned)grid, threads, smem, s>>>(c.u, (R*)c.rbar, (R*)c.trace, c.st, c.ma,
-                                                                    PP<R>::get(c), PP<R>::tab(c), c.slot);
-    }
+    const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;
+    const long long grid = std::min(ntiles, (long long)c.sms * vol_occupancy());
+    k_volume_lanes<EQ, N, R><<<(unsigned)grid, LL::THREADS, PL::bytes(), s>>>(
+        c.u, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
     return cudaGetLastError();
   }
   static cudaError_t volume_stage(const LaunchCtx& c, cudaStream_t s, const double* u_in, int first) {
-    if constexpr (kLanes) {
-      const long long ntiles = (c.ma.E + 31) / 32;
-      const long long grid = std::min(ntiles, (long long)c.sms * vol_stage_occupancy());
-      k_volume_lanes_stage<EQ, N, R><<<(unsigned)grid, LL::THREADS, PL::bytes(), s>>>(
-          u_in, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, first);
-    } else {
-      const long long grid = (c.ma.E + c.epb - 1) / c.epb;
-      const int threads = c.epb * L::NF;
-      const size_t smem = (size_t)c.epb * L::bytes_per_elem();
-      k_volume_tile_stage<EQ, N, R><<<(unsigned)grid, threads, smem, s>>>(
-          u_in, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, first);
-    }
+    const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;
+    const long long grid = std::min(ntiles, (long long)c.sms * vol_stage_occupancy());
+    k_volume_lanes_stage<EQ, N, R><<<(unsigned)grid, LL::THREADS, PL::bytes(), s>>>(
+        u_in, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, first);
     return cudaGetLastError();
   }
   static int vol_stage_occupancy() {
     static int occ = -1;
     if (occ < 0) {
       int nb = 0;
-      if constexpr (kLanes) {
-        cudaFuncSetAttribute(k_volume_lanes_stage<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)PL::bytes());
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes_stage<EQ, N, R>, LL::THREADS, PL::bytes());
-      }
+      cudaFuncSetAttribute(k_volume_lanes_stage<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)PL::bytes());
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes_stage<EQ, N, R>, LL::THREADS, PL::bytes());
       occ = nb > 0 ? nb : 1;
     }
     return occ;
   }
-  using FL = FaceLaneLayout<EQ, N, R>;
-  static constexpr bool kFaceLanes = FL::fits();
+  static unsigned face_tiles(const LaunchCtx& c) { return (unsigned)((c.ma.E + FL::EPB - 1) / FL::EPB); }
   static cudaError_t face_stage(const LaunchCtx& c, cudaStream_t s, int j, int ns) {
     const RkStage<R> rk{(R*)c.kbuf, j == ns - 1 ? c.u : c.ustage, j, ns};
-    if constexpr (kFaceLanes) {
-      const unsigned grid = (unsigned)((c.ma.E + 31) / 32);
-      k_face_stage_lanes<EQ, N, R><<<grid, FL::THREADS, FL::bytes(), s>>>(
-          c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, rk);
-    } else {
-      const long long total = c.ma.E * L::NP;
-      const unsigned grid = (unsigned)((total + 255) / 256);
-      k_face_stage<EQ, N, R><<<grid, 256, 0, s>>>(c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma,
-                                                   PP<R>::get(c), PP<R>::tab(c), c.slot, rk);
-    }
+    k_face_stage_lanes<EQ, N, R><<<face_tiles(c), FL::THREADS, FL::bytes(), s>>>(
+        c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, rk);
     return cudaGetLastError();
   }
-  static constexpr bool kBatched = EQ::DIM == 2 && !EQ::NC && kLanes && kFaceLanes;
+  static constexpr bool kBatched = EQ::DIM == 2 && !EQ::NC;
+  static_assert(!kBatched || (LL::EPB == 32 && FL::EPB == 32), "the work list holds 32-element tiles");
   static cudaError_t face_update(const LaunchCtx& c, cudaStream_t s) {
-    if constexpr (kFaceLanes) {
-      const unsigned grid = (unsigned)((c.ma.E + 31) / 32);
-      k_face_update_lanes<EQ, N, R><<<grid, FL::THREADS, FL::bytes(), s>>>(
-          c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
-    } else {
-      const long long total = c.ma.E * L::NP;
-      const unsigned grid = (unsigned)((total + 255) / 256);
-      k_face_update<EQ, N, R><<<grid, 256, 0, s>>>(c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma,
-                                                    PP<R>::get(c), PP<R>::tab(c), c.slot);
-    }
+    k_face_update_lanes<EQ, N, R><<<face_tiles(c), FL::THREADS, FL::bytes(), s>>>(
+        c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
     return cudaGetLastError();
   }
-  static constexpr bool kVolInd = kLanes && !EQ::NC && sizeof(R) == 4;
+  static constexpr bool kVolInd = !EQ::NC && sizeof(R) == 4;
   static cudaError_t volume_ind(const LaunchCtx& c, cudaStream_t s) {
     if constexpr (kVolInd) {
       static int occ = -1;
@@ -131,7 +94,7 @@ struct Variant {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes_ind<EQ, N, R>, LL::THREADS, PL::bytes());
         occ = nb > 0 ? nb : 1;
       }
-      const long long ntiles = (c.ma.E + 31) / 32;
+      const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;
       const long long grid = std::min(ntiles, (long long)c.sms * occ);
       k_volume_lanes_ind<EQ, N, R><<<(unsigned)grid, LL::THREADS, PL::bytes(), s>>>(
           c.u, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, c.araw, c.tcount, c.lt);
@@ -161,31 +124,27 @@ struct Variant {
     return cudaErrorNotSupported;
   }
   // the limited face / update part: the lane kernel for the elements the
-  // limiter does not touch, the per-node limited kernel for the others (all
-  // elements where the lane layout does not fit)
+  // limiter does not touch, the per-node limited kernel for the others
   static cudaError_t face_limited(const LaunchCtx& c, cudaStream_t s) {
     if constexpr (!EQ::NC) {
-      if constexpr (kFaceLanes) {
-        const unsigned tiles = (unsigned)((c.ma.E + 31) / 32);
-        k_face_update_lanes_clean<EQ, N, R><<<tiles, FL::THREADS, FL::bytes(), s>>>(
-            c.u, c.u_next, (const R*)c.rbar, (const R*)c.trace, c.touched, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c),
-            c.slot);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-      }
-      // over the touched elements' nodes (their number is known on the device
-      // only: a grid of four CTAs per SM strides over them), else over all nodes
-      const long long total = c.ma.E * L::NP;
-      const unsigned grid = (unsigned)std::min((total + 255) / 256, kFaceLanes ? 4LL * c.sms : (total + 255) / 256);
+      k_face_update_lanes_clean<EQ, N, R><<<face_tiles(c), FL::THREADS, FL::bytes(), s>>>(
+          c.u, c.u_next, (const R*)c.rbar, (const R*)c.trace, c.touched, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c),
+          c.slot);
+      cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+      // their number is known on the device only: a grid of four CTAs per SM
+      // strides over the touched elements' nodes
+      const long long total = c.ma.E * LL::NP;
+      const unsigned grid = (unsigned)std::min((total + 255) / 256, 4LL * c.sms);
       k_face_update_limited<EQ, N, R><<<grid, 256, 0, s>>>(c.u, c.u_next, (const R*)c.rbar, (const R*)c.trace, c.alpha,
                                                            c.tlist, c.tcount, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c),
-                                                           c.lt, c.slot, kFaceLanes ? 1 : 0);
+                                                           c.lt, c.slot);
       return cudaGetLastError();
     }
     return cudaErrorNotSupported;
   }
   using FU = FusedLayout<EQ, N, R>;
-  static constexpr bool kFused = FU::fits() && !EQ::NC;
+  static constexpr bool kFused = FU::fits() && !EQ::NC && LL::EPB == 32;
   static int fused_occupancy() {
     static int occ = -1;
     if (occ < 0) {
@@ -202,7 +161,7 @@ struct Variant {
     if constexpr (kFused) {
       const int occ = fused_occupancy();
       if (occ < 1) return cudaErrorInvalidConfiguration;
-      const long long ntiles = (c.ma.E + 31) / 32;
+      const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;
       // cooperative: every CTA resident, so the bounded readiness waits end
       const long long grid = std::min(ntiles, (long long)c.sms * occ);
       cudaLaunchConfig_t cfg = {};
@@ -221,60 +180,39 @@ struct Variant {
     return cudaErrorNotSupported;
   }
   static cudaError_t lambda(const LaunchCtx& c, cudaStream_t s) {
-    const long long total = c.ma.E * L::NP;
+    const long long total = c.ma.E * LL::NP;
     const unsigned grid = (unsigned)((total + 255) / 256);
     k_lambda<EQ, N, R><<<grid, 256, 0, s>>>(c.u, c.st, c.ma, c.slot);
     return cudaGetLastError();
   }
   static cudaError_t totals(const LaunchCtx& c, cudaStream_t s) {
-    const long long total = c.ma.E * L::NP;
+    const long long total = c.ma.E * LL::NP;
     const unsigned grid = (unsigned)((total + 255) / 256);
     k_totals<EQ, N><<<grid, 256, 0, s>>>(c.u, c.totals_part, c.ma, c.tb64);
     return cudaGetLastError();
   }
-  static cudaError_t set_smem(size_t bytes) {
-    if constexpr (kFaceLanes) {
-      cudaError_t e = cudaFuncSetAttribute(k_face_update_lanes<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)FL::bytes());
-      if (e != cudaSuccess) return e;
-      e = cudaFuncSetAttribute(k_face_stage_lanes<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               (int)FL::bytes());
-      if (e != cudaSuccess) return e;
-      if constexpr (!EQ::NC) {
-        e = cudaFuncSetAttribute(k_face_update_lanes_clean<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)FL::bytes());
-        if (e != cudaSuccess) return e;
-      }
-      if constexpr (kBatched) {
-        e = cudaFuncSetAttribute(k_face_batched<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)FL::bytes());
-        if (e != cudaSuccess) return e;
-      }
+  template <class K>
+  static cudaError_t allow(K k, size_t bytes) {
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  }
+  // dynamic shared memory of every kernel of the variant
+  static cudaError_t set_smem() {
+    cudaError_t e = allow(k_volume_lanes<EQ, N, R>, PL::bytes());
+    if (e == cudaSuccess) e = allow(k_volume_lanes_stage<EQ, N, R>, PL::bytes());
+    if (e == cudaSuccess) e = allow(k_face_update_lanes<EQ, N, R>, FL::bytes());
+    if (e == cudaSuccess) e = allow(k_face_stage_lanes<EQ, N, R>, FL::bytes());
+    if constexpr (!EQ::NC) {
+      if (e == cudaSuccess) e = allow(k_face_update_lanes_clean<EQ, N, R>, FL::bytes());
+    }
+    if constexpr (kBatched) {
+      if (e == cudaSuccess) e = allow(k_volume_batched<EQ, N, R, 0>, PL::bytes());
+      if (e == cudaSuccess) e = allow(k_volume_batched<EQ, N, R, 1>, PL::bytes());
+      if (e == cudaSuccess) e = allow(k_face_batched<EQ, N, R>, FL::bytes());
     }
     if constexpr (kFused) {
-      cudaError_t e = cudaFuncSetAttribute(k_step_fused<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)FU::bytes());
-      if (e != cudaSuccess) return e;
+      if (e == cudaSuccess) e = allow(k_step_fused<EQ, N, R>, FU::bytes());
     }
-    if constexpr (kLanes) {
-      if constexpr (kBatched) {
-        cudaError_t e = cudaFuncSetAttribute(k_volume_batched<EQ, N, R, 0>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::bytes());
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(k_volume_batched<EQ, N, R, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)PL::bytes());
-        if (e != cudaSuccess) return e;
-      }
-      cudaError_t e = cudaFuncSetAttribute(k_volume_lanes_stage<EQ, N, R>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-      if (e != cudaSuccess) return e;
-      return cudaFuncSetAttribute(k_volume_lanes<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    } else {
-      cudaError_t e = cudaFuncSetAttribute(k_volume_tile_stage<EQ, N, R>,
-                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-      if (e != cudaSuccess) return e;
-      return cudaFuncSetAttribute(k_volume_tile<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    }
+    return e;
   }
   static cudaError_t vol_batched(const BatchLaunch& b, cudaStream_t s) {
     if constexpr (kBatched) {
@@ -315,16 +253,14 @@ struct Variant {
     o->occupancy = kBatched ? &occupancy : nullptr;
     o->vol_shapes = kBatched ? 2 : 0;
     o->threads_vol = LL::THREADS;
-    o->threads_face = kFaceLanes ? FL::THREADS : 0;
+    o->threads_face = FL::THREADS;
     o->M = EQ::M;
-    o->NP = L::NP;
-    o->NF = L::NF;
+    o->NP = LL::NP;
+    o->NF = LL::NF;
     o->C = trace_comps<EQ>();
     o->ncs_per_elem = EQ::NCS ? ncs_values_per_elem<EQ, N>() : 0;
     o->dim = EQ::DIM;
-    o->vol_bytes_per_elem = L::bytes_per_elem();
-    o->lanes = kLanes;
-    o->vol_smem = &vol_smem;
+    o->lane_elems = LL::EPB;
     o->real_bytes = sizeof(R);
     o->volume = &volume;
     o->face_update = &face_update;

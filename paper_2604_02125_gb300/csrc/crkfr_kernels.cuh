@@ -1,31 +1,19 @@
-// crkfr_kernels.cuh -- shared pieces of the cRKFR step kernels on sm_103a,
-// and the general (tile-form) kernels that serve the variants whose lane form
-// (crkfr_volume_lanes.cuh) does not fit in shared memory.
+// crkfr_kernels.cuh -- shared pieces of the cRKFR step kernels on sm_103a (the
+// step's kernels are in crkfr_volume_lanes.cuh):
 //
-//  k_volume_tile  element-local cRK stages (eq. crkfr.inner) with the
-//                 flux-differencing local residual (Sec. 3, eqs.
-//                 entropy.cons.flux.dev, entropy.cons.noncons.dev), the
-//                 b-weighted volume residual of the final update (Sec. 3,
-//                 time-averaged flux differencing), and the face traces of the
-//                 time averages U, F (eq. disc.avg.flux), F^nc (Sec. 2.3) and
-//                 of lambda(u^n).  One CTA holds `epb` elements in shared
-//                 memory; one thread per line (N+1 nodes along a direction).
-//  k_face_update  the single inter-element step, one thread per node: per face
-//                 node one time-averaged Rusanov flux (eq. numflux.cons) and
-//                 the reduced-communication non-conservative flux
-//                 B(u^{n,+-}) g^avg(U) (Sec. 2.3), applied through the g2
-//                 correction derivatives g_R'(1) = 1/w_N, g_L'(0) = -1/w_0
-//                 (GLL + g2) in the FP64 update (eq. crkfr.non.cons.final);
-//                 then the CFL reduction of the new state and the
-//                 physicality flag.
+//  line_differences  flux differencing along one line (Sec. 3, eqs.
+//                 entropy.cons.flux.dev, entropy.cons.noncons.dev)
+//  face_jump      the jump of one face node: one time-averaged Rusanov flux
+//                 (eq. numflux.cons) and the reduced-communication
+//                 non-conservative flux B(u^{n,+-}) g^avg(U) (Sec. 2.3)
 //  k_lambda       CFL reduction of a state (first step after set_state).
 //  k_totals       FP64 quadrature-weighted totals (diagnostics).
-// Shared: the mesh and reference-element parameters, the step record and its
+// and the mesh and reference-element parameters, the step record and its
 // fence-free CFL protocol (reduce_lambda / step_begin), element coordinates
-// and periodic neighbours, the face-record layout and the Rusanov jump.
+// and periodic neighbours, the face-record layout.
 //
 // Layouts in HBM:
-//   u     [M][E][NP] FP64        state, updated in place by k_face_update
+//   u     [M][E][NP] FP64        state, updated in place by the face / update kernel
 //   rbar  [M][E][NP] R           sum_i b_i R(u^(i))
 //   trace [DIM][2][NF][C][E] R   face data; side 0 = xi_d = 0 face, side 1 = xi_d = 1;
 //         per face node C components, each contiguous over the elements
@@ -245,21 +233,6 @@ __device__ __forceinline__ void write_stage_prims(R* __restrict__ trace, int d, 
   }
 }
 
-template <class EQ, int N, typename R>
-struct VolLayout {
-  static constexpr int DIM = EQ::DIM, M = EQ::M, P = EQ::P, n = N + 1;
-  static constexpr int NP = ipow(n, DIM), NF = NP / n, S = rk_stages(N);
-  static constexpr int O_U0 = 0;
-  static constexpr int O_Q = O_U0 + M * NP;
-  static constexpr int O_RS = O_Q + P * NP;
-  static constexpr int O_UB = O_RS + S * M * NP;
-  static constexpr int O_FB = O_UB + M * NP;
-  static constexpr int O_FN = O_FB + DIM * M * NP;
-  static constexpr int O_LAM = O_FN + (EQ::NC ? DIM * M * NP : 0);
-  static constexpr int SZ = O_LAM + DIM * NP;    // elements of R per mesh element
-  static constexpr size_t bytes_per_elem() { return sizeof(R) * (size_t)SZ; }
-};
-
 // node index of the first node of line l in direction d, and its stride
 template <int n>
 __device__ __forceinline__ int line_base(int l, int stride) { return (l % stride) + (l / stride) * stride * n; }
@@ -364,205 +337,6 @@ __device__ __forceinline__ void line_differences(int d, const R (&q)[N + 1][EQ::
   }
 }
 
-// ---------------------------------------------------------------------------
-// Volume kernel, tile form: one CTA holds epb elements; one thread per line.
-// Used where the lane form below does not fit in shared memory.
-// ---------------------------------------------------------------------------
-// S1 = 1: a single stage with b = 1 (R-bar = R(u), face records of u), the
-// volume part of one stage of the multi-stage RKFR step; first = false takes
-// the dt the step's first launch recorded.
-template <class EQ, int N, typename R, int S1>
-__device__ __forceinline__ void volume_tile_body(const double* __restrict__ u, R* __restrict__ rbar,
-                                                 R* __restrict__ trace, DevState* __restrict__ st, const MeshArgs& ma,
-                                                 const PhysParams<R>& pp, const RefTab<R>& tb, int slot, bool first) {
-  using L = VolLayout<EQ, N, R>;
-  constexpr int DIM = L::DIM, M = L::M, P = L::P, n = L::n, NP = L::NP, NF = L::NF, S = S1 ? S1 : L::S;
-  constexpr int C = trace_comps<EQ>();
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  R* sm = reinterpret_cast<R*>(smem_raw);
-
-  const int NT = blockDim.x;
-  const int epb = NT / NF;
-  const int tid = threadIdx.x;
-  const long long E = ma.E;
-  const long long e0 = (long long)blockIdx.x * epb;
-  const int nel = (int)min((long long)epb, E - e0);
-  const int el = tid / NF, l = tid % NF;
-  const bool active = el < nel;
-  R* my = sm + (size_t)el * L::SZ;
-
-  __shared__ double s_dt;
-  if (tid == 0) s_dt = first ? step_begin(st, slot, ma.cfl, ma.dt_fixed, blockIdx.x == 0) : st->dt;
-  __syncthreads();
-  const R dtR = dt_as<R>(s_dt);
-
-  // u^n -> shared memory (coalesced over [v][e0..e0+nel)[p])
-#pragma unroll 1
-  for (int v = 0; v < M; ++v)
-    for (int r = tid; r < nel * NP; r += NT) {
-      const int ee = r / NP, p = r % NP;
-      sm[(size_t)ee * L::SZ + L::O_U0 + v * NP + p] = (R)u[((size_t)v * E + e0) * NP + r];
-    }
-  __syncthreads();
-
-#pragma unroll
-  for (int i = 0; i < S; ++i) {
-    // ---- node phase: stage state u^(i), pair data, time-average face sums
-    if (active) {
-#pragma unroll
-      for (int k = 0; k < n; ++k) {
-        const int p = l * n + k;
-        R uu[M];
-#pragma unroll
-        for (int v = 0; v < M; ++v) {
-          R acc = R(0);
-#pragma unroll
-          for (int j = 0; j < i; ++j)
-            if (rk_a(N, i, j) != 0.0) acc += R(rk_a(N, i, j)) * my[L::O_RS + (j * M + v) * NP + p];
-          uu[v] = my[L::O_U0 + v * NP + p] - dtR * acc;
-        }
-        R q[P];
-        EQ::pair_data(uu, q, pp);
-#pragma unroll
-        for (int c = 0; c < P; ++c) my[L::O_Q + c * NP + p] = q[c];
-        if constexpr (EQ::NCS) {
-          // face traces of this stage (stage-wise non-conservative flux)
-          int rq = p;
-#pragma unroll
-          for (int d = 0; d < DIM; ++d) {
-            const int cq = rq % n;
-            rq /= n;
-            const int stride = ipow(n, d);
-            if (cq == 0 || cq == N)
-              write_stage_prims<EQ, N, R>(trace, d, cq == N ? 1 : 0, (p % stride) + (p / (stride * n)) * stride, i, E,
-                                          e0 + el, q);
-          }
-        }
-#pragma unroll
-        for (int v = 0; v < M; ++v) my[L::O_RS + (i * M + v) * NP + p] = R(0);
-        // which faces this node lies on
-        int rem = p;
-        bool onface = false;
-        int cd[3] = {0, 0, 0};
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) { cd[d] = rem % n; rem /= n; onface = onface || cd[d] == 0 || cd[d] == N; }
-        if (i == 0) {
-#pragma unroll
-          for (int d = 0; d < DIM; ++d)
-            if (cd[d] == 0 || cd[d] == N) my[L::O_LAM + d * NP + p] = EQ::wave_speed(d, q, pp);
-        }
-        const double bi = S1 ? 1.0 : rk_b(N, i);
-        if (bi != 0.0 && onface) {
-          const R b = R(bi);
-#pragma unroll
-          for (int v = 0; v < M; ++v) {
-            R* ub = &my[L::O_UB + v * NP + p];
-            *ub = (i == 0 ? R(0) : *ub) + b * uu[v];
-          }
-#pragma unroll
-          for (int d = 0; d < DIM; ++d) {
-            if (cd[d] == 0 || cd[d] == N) {
-              R f[M];
-              EQ::flux(d, q, f, pp);
-#pragma unroll
-              for (int v = 0; v < M; ++v) {
-                R* fb = &my[L::O_FB + (d * M + v) * NP + p];
-                *fb = (i == 0 ? R(0) : *fb) + b * f[v];
-              }
-              if constexpr (EQ::NC) {
-                R g[2], nc[M];
-#pragma unroll
-                for (int v = 0; v < M; ++v) nc[v] = R(0);
-                EQ::ncg(d, q, g);
-                EQ::nc_apply(d, q, g, nc);
-#pragma unroll
-                for (int v = 0; v < M; ++v) {
-                  R* fn = &my[L::O_FN + (d * M + v) * NP + p];
-                  *fn = (i == 0 ? R(0) : *fn) + b * nc[v];
-                }
-              }
-            }
-          }
-        }
-      }
-    }
-    __syncthreads();
-
-    // ---- line phase: flux differencing along each direction
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-      if (active) {
-        constexpr int dummy = 0;
-        (void)dummy;
-        const int stride = ipow(n, d);
-        const int base = line_base<n>(l, stride);
-        R q[n][P];
-#pragma unroll
-        for (int k = 0; k < n; ++k)
-#pragma unroll
-          for (int c = 0; c < P; ++c) q[k][c] = my[L::O_Q + c * NP + base + k * stride];
-        R acc[n][M];
-        R fend[2][M];
-        line_differences<EQ, N, R, true>(d, q, acc, fend, pp, tb, d, R(1));
-#pragma unroll
-        for (int k = 0; k < n; ++k)
-#pragma unroll
-          for (int v = 0; v < M; ++v) my[L::O_RS + (i * M + v) * NP + base + k * stride] += acc[k][v];
-      }
-      __syncthreads();
-    }
-  }
-
-  // ---- outputs: Rbar = sum_i b_i R_i (coalesced over [v][elements][p])
-#pragma unroll 1
-  for (int v = 0; v < M; ++v)
-    for (int r = tid; r < nel * NP; r += NT) {
-      const int ee = r / NP, p = r % NP;
-      const R* mm = sm + (size_t)ee * L::SZ;
-      R s = R(0);
-#pragma unroll
-      for (int i = 0; i < S; ++i)
-        if ((S1 ? 1.0 : rk_b(N, i)) != 0.0) s += R(S1 ? 1.0 : rk_b(N, i)) * mm[L::O_RS + (i * M + v) * NP + p];
-      rbar[((size_t)v * E + e0) * NP + r] = s;
-    }
-  // face traces: per face node C components (coalesced over the elements)
-#pragma unroll 1
-  for (int ds = 0; ds < DIM * 2; ++ds)
-    for (int idx = tid; idx < nel * NF * C; idx += NT) {
-    const int ee = idx % nel;
-    const int c = (idx / nel) % C;
-    const int f = idx / (nel * C);
-    const int side = ds & 1;
-    const int d = ds >> 1;
-    const int stride = ipow(n, d);
-    const int p = line_base<n>(f, stride) + side * N * stride;
-    const R* mm = sm + (size_t)ee * L::SZ;
-    R val;
-    if (c < M) val = mm[L::O_UB + c * NP + p];
-    else if (c < 2 * M) val = mm[L::O_FB + (d * M + (c - M)) * NP + p];
-    else if (c == 2 * M) val = mm[L::O_LAM + d * NP + p];
-    else if (c < 3 * M + 1) val = mm[L::O_FN + (d * M + (c - 2 * M - 1)) * NP + p];
-    else val = mm[L::O_U0 + (c - 3 * M - 1) * NP + p];
-    trace[trace_index<EQ, NF>(d, side, f, c, E, e0 + ee)] = val;
-  }
-}
-
-template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(256)
-k_volume_tile(const double* __restrict__ u, R* __restrict__ rbar, R* __restrict__ trace,
-         DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb, int slot) {
-  volume_tile_body<EQ, N, R, 0>(u, rbar, trace, st, ma, pp, tb, slot, true);
-}
-
-// volume part of one RKFR stage (input: the stage state)
-template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(256)
-k_volume_tile_stage(const double* __restrict__ u, R* __restrict__ rbar, R* __restrict__ trace,
-                    DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
-                    int slot, int first) {
-  volume_tile_body<EQ, N, R, 1>(u, rbar, trace, st, ma, pp, tb, slot, first != 0);
-}
-
 // physicality and sum_d lambda_d/dx_d of an updated state; the FP32 form
 // evaluates the wave speeds in FP32 (the dt reduction is a max)
 template <class EQ, typename R>
@@ -617,9 +391,6 @@ __device__ __forceinline__ void wave_speeds_fp64(bool on, const double* uu, cons
   }
 }
 
-// ---------------------------------------------------------------------------
-// Face + update kernel: one thread per node
-// ---------------------------------------------------------------------------
 // the C components of the record of face node f of face (d, side) of element e
 template <class EQ, int N, typename R, bool COH = false>
 __device__ __forceinline__ void load_face_record(const R* __restrict__ trace, long long E, int d, int side, int f,
@@ -692,111 +463,8 @@ __device__ __forceinline__ void face_jump(const R* __restrict__ trace, long long
   }
 }
 
-// RK = true: stage mode of the multi-stage RKFR step (RkStage)
-template <class EQ, int N, typename R, bool RK>
-__device__ __forceinline__ void face_update_body(double* __restrict__ u, const R* __restrict__ rbar,
-                                                 const R* __restrict__ trace, DevState* __restrict__ st,
-                                                 const MeshArgs& ma, const PhysParams<R>& pp, const RefTab<R>& tb,
-                                                 int slot, const RkStage<R>& rk) {
-  constexpr int DIM = EQ::DIM, M = EQ::M, n = N + 1, NP = ipow(n, DIM);
-  constexpr bool F32 = sizeof(R) == 4;
-  const long long E = ma.E;
-  // a volume CTA that timed out left its records unwritten: leave u^n as it is
-  if (st->status & ST_TIMEOUT) return;
-  const unsigned gid = blockIdx.x * blockDim.x + threadIdx.x;
-  R lam = R(0);
-  bool bad = false;
-  if (gid < (unsigned)(E * NP)) {
-    const unsigned e = gid / NP;
-    const int p = (int)(gid % NP);
-    unsigned ec[3] = {0, 0, 0};
-    elem_coords<DIM>(e, ma, ec);
-    const R dtR = step_dt<R>(st);
-    // increment of the final update (eq. crkfr.non.cons.final) in the path's
-    // arithmetic: -dt Rbar - dt J^- g_R'(1)/dx + dt J^+ (-g_L'(0))/dx
-    R du[M];
-#pragma unroll
-    for (int v = 0; v < M; ++v) du[v] = -dtR * rbar[((size_t)v * E + e) * NP + p];
-    int rem = p;
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-      const int cd = rem % n;
-      rem /= n;
-      const int stride = ipow(n, d);
-      const int f = (p % stride) + (p / (stride * n)) * stride;
-      if (cd == N) {   // face xi_d = 1: element is the '-' state
-        const unsigned nb = neighbour_of(e, ec, d, +1, ma);
-        R J[M];
-        face_jump<EQ, N, R>(trace, E, d, 1, e, nb, f, J, pp, tb);
-        const R s = dtR * tb.iwN * inv_dx_of<R>(ma, d);
-#pragma unroll
-        for (int v = 0; v < M; ++v) du[v] -= s * J[v];
-      }
-      if (cd == 0) {   // face xi_d = 0: element is the '+' state
-        const unsigned nb = neighbour_of(e, ec, d, -1, ma);
-        R J[M];
-        face_jump<EQ, N, R>(trace, E, d, 0, e, nb, f, J, pp, tb);
-        const R s = dtR * tb.iw0 * inv_dx_of<R>(ma, d);
-#pragma unroll
-        for (int v = 0; v < M; ++v) du[v] += s * J[v];
-      }
-    }
-    bool last = true;
-    double* dst = u;
-    if constexpr (RK) {
-      // du is this stage's K_j; combine it with the earlier stages' (eq. rkfr1
-      // for the next stage state, eq. rkfr2 at the last stage)
-      last = rk.j == rk.s - 1;
-      const size_t nodes = (size_t)E * NP;
-#pragma unroll
-      for (int v = 0; v < M; ++v) {
-        const size_t g = ((size_t)v * E + e) * NP + p;
-        const R kj = du[v];
-        if (!last) rk.k[(size_t)rk.j * M * nodes + g] = kj;
-        R acc = (last ? tb.b[rk.j] : tb.a[rk.j + 1][rk.j]) * kj;
-        for (int q = 0; q < rk.j; ++q) {
-          const R c = last ? tb.b[q] : tb.a[rk.j + 1][q];
-          if (c != R(0)) acc += c * rk.k[(size_t)q * M * nodes + g];
-        }
-        du[v] = acc;
-      }
-      if (!last) dst = rk.uout;
-    }
-    // u^{n+1} = u^n + du in FP64 (one FP64 add per variable)
-    double uu[M];
-#pragma unroll
-    for (int v = 0; v < M; ++v) {
-      const size_t g = ((size_t)v * E + e) * NP + p;
-      if constexpr (F32) uu[v] = u[g] + f2d_int(du[v]);
-      else uu[v] = u[g] + du[v];
-      dst[g] = uu[v];
-    }
-    if (last) bad = !physical_state<EQ, R>(uu, ma, lam);
-  }
-  // the CFL reduction of the new state (RKFR: after the last stage only; the
-  // stage index is uniform over the grid)
-  if (!RK || rk.j == rk.s - 1) reduce_lambda<R>(lam, bad, st, slot ^ 1);
-}
-
-template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(256)
-k_face_update(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
-              DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
-              int slot) {
-  face_update_body<EQ, N, R, false>(u, rbar, trace, st, ma, pp, tb, slot, RkStage<R>{nullptr, nullptr, 0, 1});
-}
-
-// face / update part of stage rk.j of the multi-stage RKFR step
-template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(256)
-k_face_stage(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
-             DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
-             int slot, const RkStage<R> rk) {
-  face_update_body<EQ, N, R, true>(u, rbar, trace, st, ma, pp, tb, slot, rk);
-}
-
 // CFL reduction of the current state (used after set_state); wave speeds in
-// the path's arithmetic R, like the reduction inside k_face_update
+// the path's arithmetic R, like the reduction of the face / update kernel
 template <class EQ, int N, typename R>
 __global__ void __launch_bounds__(256)
 k_lambda(const double* __restrict__ u, DevState* __restrict__ st, const MeshArgs ma, int slot) {

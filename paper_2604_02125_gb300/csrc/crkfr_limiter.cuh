@@ -16,11 +16,10 @@
 //                        flux at element faces, the first-order subcell update
 //                        u^L with the same face flux, the blend
 //                        (1 - a_e) u^H + a_e u^L into the other state buffer,
-//                        and the CFL reduction of the result.  Where the lane
-//                        face kernel exists it takes the elements the limiter
-//                        does not touch (a = 0 there and at every face
-//                        neighbour: the plain update, k_face_update_lanes_clean)
-//                        and this kernel only the others.
+//                        and the CFL reduction of the result, for the elements
+//                        the limiter touches; the others (a = 0 there and at
+//                        every face neighbour) take the plain update
+//                        (k_face_update_lanes_clean).
 //
 // The limited face flux at a face node between elements '-' and '+':
 //   F_blend = (1 - a_f) F^num + a_f f_lo   (f_lo alone where a_f = 1),
@@ -436,9 +435,8 @@ __device__ __forceinline__ void limited_face_flux(const double* __restrict__ uin
 }
 
 // ---------------------------------------------------------------------------
-// Limited face / update kernel: one thread per node (alpha: the smoothed
-// coefficients; only_touched: leave the elements the limiter does not touch
-// to the lane kernel)
+// Limited face / update kernel: one thread per node of the elements the limiter
+// touches (alpha: the smoothed coefficients)
 // ---------------------------------------------------------------------------
 template <class EQ, int N, typename R>
 __global__ void __launch_bounds__(256)
@@ -446,17 +444,16 @@ k_face_update_limited(const double* __restrict__ uin, double* __restrict__ uout,
                       const R* __restrict__ trace, const double* __restrict__ alpha,
                       const unsigned* __restrict__ tlist, const unsigned* __restrict__ tcount,
                       DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
-                      const LimTab lt, int slot, int only_touched) {
+                      const LimTab lt, int slot) {
   constexpr int DIM = EQ::DIM, M = EQ::M, n = N + 1, NP = ipow(n, DIM), NF = NP / n;
   constexpr bool F32 = sizeof(R) == 4;
   const long long E = ma.E;
   if (st->status & ST_TIMEOUT) return;
   R lam = R(0);
   bool bad = false;
-  // nodes of the touched elements (only_touched), else of every element
-  const unsigned total = (only_touched ? *tcount : (unsigned)E) * (unsigned)NP;
+  const unsigned total = *tcount * (unsigned)NP;   // nodes of the touched elements
   for (unsigned gid = blockIdx.x * blockDim.x + threadIdx.x; gid < total; gid += gridDim.x * blockDim.x) {
-    const unsigned e = only_touched ? tlist[gid / NP] : gid / NP;
+    const unsigned e = tlist[gid / NP];
     const int p = (int)(gid % NP);
     unsigned ec[3] = {0, 0, 0};
     elem_coords<DIM>(e, ma, ec);

@@ -2,16 +2,16 @@
 // the persistent volume kernel (single solve and batched), the face/update
 // kernel (single solve and batched) and their shared-memory layouts.
 //
-// Same computation as k_volume_tile (element-local cRK stages with the
-// flux-differencing residual, the b-weighted volume residual and the face
-// traces of the time averages; eqs. crkfr.inner, entropy.cons.flux.dev,
-// entropy.cons.noncons.dev, disc.avg.flux), mapped for throughput:
+// Volume: element-local cRK stages with the flux-differencing residual, the
+// b-weighted volume residual and the face traces of the time averages (eqs.
+// crkfr.inner, entropy.cons.flux.dev, entropy.cons.noncons.dev,
+// disc.avg.flux), mapped for throughput:
 //
-//  * a CTA holds 32 elements; warp w handles line index w of every element
-//    and lane l handles element l, so every shared-memory access of a warp
-//    touches 32 different elements at the same offset: with an odd element
-//    stride there are no bank conflicts, and whether a line lies on a face is
-//    uniform across the warp;
+//  * a CTA holds 32 elements (16 or 8 where the layout would not fit,
+//    LaneLayout::EPB); warp w handles line index w of every element and lane l
+//    handles element l, so every shared-memory access of a warp touches 32
+//    different elements at the same offset: with an odd element stride there
+//    are no bank conflicts;
 //  * each thread owns one x-line (N+1 nodes): u^n, the stage combination, the
 //    pair data and the whole x-direction flux differencing stay in
 //    registers; only the y (and z) lines go through shared memory;
@@ -185,17 +185,37 @@ struct LaneLayout<EQ, N, R, 0> {
   static constexpr int O_U0 = O_RY + (DIM > 1 ? M * NP : 0);   // [M][NP] u^n
   static constexpr int SZ0 = O_U0 + M * NP;
   static constexpr int SZ = SZ0 | 1;                           // odd element stride: no bank conflicts
-  static constexpr int EPB = 32;
-  static constexpr int THREADS = 32 * NF;
+  // Elements per CTA: 32 (a warp = one line of 32 elements) where the layout
+  // fits in shared memory, else 16 or 8 (a warp = 2 or 4 lines): FP64 in 3D and
+  // GLM-MHD N = 5, FP32 3D N >= 4.  Lines of different offsets in a warp can meet in a
+  // bank; in FP64 an access is served per half-warp, so 16 elements have none.
+  // us per volume launch against one thread per line with the stages in shared
+  // memory (4 to 8 warps per SM), which this replaced: 3D FP64 N = 3 22x20x19
+  // 1498 -> 1193, N = 4 14^3 3942 -> 1714, N = 5 10^3 4755 -> 1238, FP32 N = 4 32^3 3432 -> 862 (8
+  // elements; 937 with 16), N = 5 24^3 3993 -> 931 (16; 959 with 8), GLM-MHD FP64
+  // N = 5 64^2 7191 -> 1826.  3D FP32 N = 3: 1588 with 32, 1605 with 16, 1706 with 8 (64^3).
+  static constexpr size_t kSmemCta = 227 * 1024 - 16;   // the mbarrier after the layout
+  static constexpr bool fits_with(int e) { return sizeof(R) * (size_t)SZ * e <= kSmemCta && e * NF <= 1024; }
+  static constexpr int EPB = fits_with(32) ? 32 : fits_with(16) && !(DIM == 3 && N == 4) ? 16 : 8;
+  static constexpr int THREADS = EPB * NF;
+  // resident CTAs of a layout with fewer than 32 elements: what shared memory
+  // holds (with the staging buffer), up to 512 threads
+  static constexpr int small_minb() {
+    const size_t stage = sizeof(double) * (size_t)M * EPB * NP, b = bytes() + stage <= kSmemCta ? bytes() + stage : bytes();
+    const int by_smem = (int)(228 * 1024 / (b + 1040)), by_threads = 512 / THREADS;
+    const int m = by_smem < by_threads ? by_smem : by_threads;
+    return m > 1 ? m : 1;
+  }
   static constexpr size_t bytes() { return sizeof(R) * (size_t)SZ * EPB; }
   // packed x/y form (2D Euler, FP32 pair fluxes)
   static constexpr bool PACK = PackXY<EQ>::value && sizeof(R) == 4 && N <= kPackMaxN;
   // CTAs per SM the register allocation aims at (the packed form holds both
   // lines' pair data at once)
   static constexpr int MINB = EQ::NC ? (2 * (bytes() + 1024) <= 228 * 1024 ? kMinBNc : 1)
+                            : EPB < 32 ? small_minb()
                             : (THREADS <= 128) ? ((N == 2 && sizeof(R) == 4) ? kMinB2 : PACK ? kMinB3 : 4)
                             : (DIM == 2) ? (N == 4 ? (PACK ? kMinB4Pack : kMinB4) : N == 5 ? kMinB5 : 1) : 1;
-  static constexpr bool fits() { return bytes() <= 227 * 1024 && THREADS <= 1024; }
+  static constexpr bool fits() { return fits_with(EPB); }
 };
 
 template <class EQ, int N, typename R>
@@ -350,10 +370,10 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
   constexpr int NS = rk_nsaved(N) > 0 ? rk_nsaved(N) : 1;
 
   const int tid = threadIdx.x;
-  const int l = tid >> 5;              // line index (warp-uniform)
-  const int el = tid & 31;             // element within the CTA
+  const int l = tid / L::EPB;          // line index (warp-uniform with 32 elements)
+  const int el = tid % L::EPB;         // element within the CTA
   const long long E = ma.E;
-  const int nel = (int)min(32LL, E - e0);
+  const int nel = (int)min((long long)L::EPB, E - e0);
   const bool active = el < nel;
   R* my = sm + (size_t)el * L::SZ;
   constexpr bool PACK = L::PACK;
@@ -366,7 +386,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
   // each variable's 32 NP values are n rounds of the CTA's 32 NF threads:
   // the node offsets of the rounds are computed once, the variable loop only
   // adds its stride
-  static_assert(32 * NP == n * L::THREADS, "a tile's values per variable are n rounds of the CTA");
+  static_assert(L::EPB * NP == n * L::THREADS, "a tile's values per variable are n rounds of the CTA");
   int tofs[n];
   bool tok[n];
 #pragma unroll
@@ -377,7 +397,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
   }
   {
     const double* src = staged ? staged + tid : u + (size_t)e0 * NP + tid;
-    const size_t vstride = staged ? (size_t)32 * NP : (size_t)E * NP;
+    const size_t vstride = staged ? (size_t)L::EPB * NP : (size_t)E * NP;
 #pragma unroll 1
     for (int v = 0; v < M; ++v, src += vstride) {
 #pragma unroll
@@ -668,9 +688,10 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
 template <class EQ, int N, typename R>
 struct PersistLayout {
   using L = LaneLayout<EQ, N, R>;
-  static constexpr bool STAGE = !EQ::NC || kStageNc;
   static constexpr size_t O_STAGE = (L::bytes() + 15) & ~(size_t)15;
-  static constexpr size_t STAGE_BYTES = STAGE ? sizeof(double) * (size_t)EQ::M * 32 * L::NP : 0;
+  static constexpr size_t WANT = sizeof(double) * (size_t)EQ::M * L::EPB * L::NP;
+  static constexpr bool STAGE = (!EQ::NC || kStageNc) && O_STAGE + WANT + 16 <= 227 * 1024;
+  static constexpr size_t STAGE_BYTES = STAGE ? WANT : 0;
   static constexpr size_t O_BAR = O_STAGE + STAGE_BYTES;
   static constexpr size_t bytes() { return O_BAR + 16; }
   static constexpr bool fits() { return L::fits() && bytes() <= 227 * 1024; }
@@ -693,16 +714,16 @@ __device__ __forceinline__ void volume_lanes_persistent(const double* __restrict
                                                         const RefTab<R>& tb, int slot, bool first,
                                                         After after_tile = After{}) {
   using PL = PersistLayout<EQ, N, R>;
-  constexpr int M = EQ::M, NP = LaneLayout<EQ, N, R>::NP;
+  constexpr int M = EQ::M, NP = LaneLayout<EQ, N, R>::NP, EPB = LaneLayout<EQ, N, R>::EPB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R* sm = reinterpret_cast<R*>(smem_raw);
   double* staging = reinterpret_cast<double*>(smem_raw + PL::O_STAGE);
   unsigned long long* bar = reinterpret_cast<unsigned long long*>(smem_raw + PL::O_BAR);
   const long long E = ma.E;
-  const unsigned ntiles = (unsigned)((E + 31) / 32);
-  auto whole = [&](unsigned t) { return PL::STAGE && ma.tma_ok && (long long)(t + 1) * 32 <= E; };
+  const unsigned ntiles = (unsigned)((E + EPB - 1) / EPB);
+  auto whole = [&](unsigned t) { return PL::STAGE && ma.tma_ok && (long long)(t + 1) * EPB <= E; };
   auto pf_of = [&](unsigned t) {
-    return Prefetch{u + (size_t)t * 32 * NP, E * NP, (unsigned)(32 * NP * sizeof(double)), staging, bar};
+    return Prefetch{u + (size_t)t * EPB * NP, E * NP, (unsigned)(EPB * NP * sizeof(double)), staging, bar};
   };
   __shared__ double s_dt;
   if (threadIdx.x == 0) {
@@ -731,11 +752,11 @@ __device__ __forceinline__ void volume_lanes_persistent(const double* __restrict
     }
     const unsigned tn = t + gridDim.x;
     const Prefetch pf = (tn < ntiles && whole(tn)) ? pf_of(tn) : Prefetch{nullptr, 0, 0, nullptr, nullptr};
-    volume_lanes_tile<EQ, N, R, 0, S1, true>(u, rbar, trace, st, ma, pp, tb, (long long)t * 32, dtR, sm,
+    volume_lanes_tile<EQ, N, R, 0, S1, true>(u, rbar, trace, st, ma, pp, tb, (long long)t * EPB, dtR, sm,
                                        staged ? staging : nullptr, pf);
     __syncthreads();   // shared memory is reused by the next tile
     if constexpr (!std::is_same<After, NoTileWork>::value) {
-      after_tile((long long)t * 32, reinterpret_cast<const float*>(sm));
+      after_tile((long long)t * EPB, reinterpret_cast<const float*>(sm));
       __syncthreads();
     }
   }
@@ -768,8 +789,8 @@ k_volume_lanes_ind(const double* __restrict__ u, R* __restrict__ rbar, R* __rest
   if (blockIdx.x == 0 && threadIdx.x == 0) *tcount = 0u;
   auto indicator = [&](long long e0, const float* sm) {
     float* smw = const_cast<float*>(sm);
-    const int tid = threadIdx.x, l = tid >> 5, el = tid & 31;
-    const int nel = (int)min(32LL, ma.E - e0);
+    const int tid = threadIdx.x, l = tid / L::EPB, el = tid % L::EPB;
+    const int nel = (int)min((long long)L::EPB, ma.E - e0);
     float* my = smw + (size_t)el * L::SZ;
     if (el < nel) {
       const float gm1 = ma.gamma_f - 1.0f;
@@ -787,7 +808,7 @@ k_volume_lanes_ind(const double* __restrict__ u, R* __restrict__ rbar, R* __rest
       }
     }
     __syncthreads();
-    if (tid < 32 && el < nel) {
+    if (tid < L::EPB && el < nel) {
       const float En = indicator_of_values<EQ, N, float>([&](int p) { return my[L::O_Q + p]; }, lt);
       const float a = alpha_of_energy_f32(En, lt);
       araw[e0 + el] = a >= 0.0f ? f2d_int(a) : -1.0;   // k_alpha_fix takes it in FP64
@@ -819,11 +840,12 @@ template <class EQ, int N, typename R>
 struct FaceLaneLayout {
   static constexpr int DIM = EQ::DIM, M = EQ::M, n = N + 1;
   static constexpr int NP = ipow(n, DIM), NF = NP / n;
-  static constexpr int THREADS = 32 * NF;
-  // scaled jumps of every face: [DIM][side][M][face node][32 elements], rows of
+  static constexpr int EPB = 32 * NF <= 1024 ? 32 : 16;   // elements per CTA (16: 3D, N = 5)
+  static constexpr int THREADS = EPB * NF;
+  // scaled jumps of every face: [DIM][side][M][face node][EPB elements], rows of
   // LD values (phase A writes a row per warp; in phase B the lanes of a warp
   // read several face nodes of few elements: 2 f + e falls into distinct banks)
-  static constexpr int LD = 34;
+  static constexpr int LD = EPB + 2;
   __host__ __device__ static constexpr int jump(int d, int side, int v) { return ((d * 2 + side) * M + v) * NF * LD; }
   static constexpr size_t bytes() { return sizeof(R) * (size_t)jump(DIM, 0, 0); }
   static constexpr bool fits() { return THREADS <= 1024 && bytes() <= 227 * 1024; }
@@ -835,14 +857,15 @@ struct FaceLaneLayout {
   // 1536 57.6 / 29.0 / 29.9 / 52 (spills); 64 batched solves 267 / 234 (1024) /
   // 221 (1152) / 228 (1280); RKFR 256^2 176 / 126 / 126 / 129.
   static constexpr int minb(int t) { return t / THREADS > 1 ? t / THREADS : 1; }
-  static constexpr int MINB = minb(sizeof(R) == 8 ? 512 : EQ::NC ? 768 : DIM == 3 ? 1536 : 1280), MINB1 = minb(1152);
+  static constexpr int MINB = minb(sizeof(R) == 8 ? 512 : EQ::NC ? 768 : DIM == 3 ? 1536 : 1280), 
+                       MINB1 = minb(sizeof(R) == 8 ? 512 : EQ::NC ? 768 : 1152);
 };
 
-// One tile of 32 elements starting at e0 (sj: the CTA's shared memory; slot:
+// One tile of EPB elements starting at e0 (sj: the CTA's shared memory; slot:
 // step parity of the CFL reduction).
 //
 // Phase A (warp = line index l, lane = element): every warp computes the Rusanov
-// jumps of face node f = l of all 2 DIM faces of its 32 elements, scaled by
+// jumps of face node f = l of all 2 DIM faces of its elements, scaled by
 // their correction factor, into shared memory: every record load is a run of 32
 // elements, the same loads for every warp.
 // Phase B (thread = node, in memory order): the tile's values of a variable are
@@ -886,14 +909,14 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
     if (st->status & ST_TIMEOUT) return;
   }
   const R dtR = FUSED ? dt_fused : step_dt<R>(st);
-  const int nel = (int)min(32LL, E - (long long)e0);
+  const int nel = (int)min((long long)L::EPB, E - (long long)e0);
   const size_t vs = (size_t)E * NP;   // values per variable
   const size_t g0 = (size_t)e0 * NP + tid;
 
   // ---- phase A: scaled jumps, -dt J^- g_R'(1)/dx at the xi = 1 faces and
   // +dt J^+ (-g_L'(0))/dx at the xi = 0 faces
   {
-    const int l = tid >> 5, el = tid & 31;
+    const int l = tid / L::EPB, el = tid % L::EPB;
     const unsigned e = e0 + el;
     if (el < nel && !(touched && touched[e])) {
       unsigned ec[3] = {0, 0, 0};
@@ -1008,7 +1031,7 @@ k_face_update_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R*
                     DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                     int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  face_lanes_tile<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * 32u, slot, reinterpret_cast<R*>(smem_raw));
+  face_lanes_tile<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot, reinterpret_cast<R*>(smem_raw));
 }
 
 // the limited step's elements that the limiter does not touch: the plain
@@ -1020,7 +1043,7 @@ k_face_update_lanes_clean(double* __restrict__ uin, double* __restrict__ uout, c
                           DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                           int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  face_lanes_tile<EQ, N, R>(uin, rbar, trace, st, ma, pp, tb, blockIdx.x * 32u, slot, reinterpret_cast<R*>(smem_raw),
+  face_lanes_tile<EQ, N, R>(uin, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot, reinterpret_cast<R*>(smem_raw),
                             RkStage<R>{nullptr, nullptr, 0, 1}, R(0), touched, uout);
 }
 
@@ -1031,7 +1054,7 @@ k_face_stage_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R* 
                    DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                    int slot, const RkStage<R> rk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  face_lanes_tile<EQ, N, R, true>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * 32u, slot,
+  face_lanes_tile<EQ, N, R, true>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot,
                                   reinterpret_cast<R*>(smem_raw), rk);
 }
 
