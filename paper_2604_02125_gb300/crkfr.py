@@ -288,8 +288,9 @@ def step_noalloc(mesh, u_in, u_out, dt_out=None, prec="fp64", dt_fixed=0.0, stre
         stream = stream.cuda_stream
     # the C entry point takes raw device pointers and trusts their sizes: check
     # type, layout, size and device here, before any kernel can touch them
-    from . import inputs
-    need = inputs.nvars(mesh) * inputs.num_elems(mesh) * inputs.nodes_per_elem(mesh)
+    need = d.dim + 2 if d.eq == EQ["euler"] else 9
+    for k in range(d.dim):
+        need *= d.cells[k] * (d.degree_N + 1)
     dev = torch.cuda.current_device()
     for name, t in (("u_in", u_in), ("u_out", u_out)):
         if not isinstance(t, torch.Tensor) or not t.is_cuda:

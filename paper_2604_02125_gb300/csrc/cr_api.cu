@@ -9,6 +9,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -126,8 +127,17 @@ bool get_ops(int eq, int dim, int prec, int vol, int N, VariantOps* o, int ncflu
 }
 
 void fill_ref_tables(int N, int eq, const MeshArgs& ma, RefTab<double>* t64, RefTab<float>* t32) {
-  double xi[6], w[6], D[6][6];
-  ref_tables(N, xi, w, D);
+  // nodes, weights and D of the degree: computed on first use (Newton's method)
+  struct Ref {
+    double xi[6], w[6], D[6][6];
+  };
+  static const std::array<Ref, 6> refs = [] {
+    std::array<Ref, 6> r{};
+    for (int k = 1; k <= 5; ++k) ref_tables(k, r[k].xi, r[k].w, r[k].D);
+    return r;
+  }();
+  const double(&w)[6] = refs[N].w;
+  const double(&D)[6][6] = refs[N].D;
   std::memset(t64, 0, sizeof(*t64));
   std::memset(t32, 0, sizeof(*t32));
   const double sa = eq == CR_EULER ? 2.0 : 0.5;   // row scale of the two-point flux (RefTab::A)

@@ -23,6 +23,7 @@ struct LaunchCtx {
   RefTab<float> tb32;
   int sms;            // multiprocessors of the device (persistent grids)
   int slot;           // step parity: CFL-reduction slot of the state the next step starts from
+  FaceOut out;        // the face / update kernel's other outputs (cr_step_noalloc)
   // multi-stage RKFR scratch: stage state u^(j) (FP64, like u) and the
   // increments K_0..K_{s-2} ([stage][var][elem][node], R)
   double* ustage;

@@ -13,13 +13,16 @@
 // The array exists once per device that loads the library and lives until the
 // process exits.  All calls on a device share it and it keeps the last call's
 // contents, so calls that overlap on the GPU (on different streams, or from
-// several threads) race; the step record is cleared at the start of every
-// call.  The array's device address is looked up on the first call on each
+// several threads) race; the step record is clean at the start of every
+// call (the face kernel zeroes the CFL slot its step has read, the first
+// kernel the status; a call whose launches failed makes the next one clear
+// it whole).  The array's device address is looked up on the first call on each
 // device and kept for the life of the process; cudaDeviceReset destroys the
 // context that address belongs to, so a process that resets a device must
 // not call this entry point on that device afterwards.
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstring>
 #include <mutex>
 
@@ -35,6 +38,23 @@ namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_mutex;
 void* g_scratch_ptr[kMaxDevices] = {nullptr};
+std::atomic<bool> g_dirty[kMaxDevices];   // the record may hold a failed call's values
+
+// The variant's kernels get their shared memory allowance on the first call per
+// device (a dozen runtime calls otherwise, of each call's host time).
+using SetSmem = cudaError_t (*)();
+constexpr int kMaxVariants = 128;   // variants per process: at most 110
+SetSmem g_ready[kMaxDevices][kMaxVariants];
+int g_nready[kMaxDevices];
+
+cudaError_t prepare_variant(int dev, SetSmem f) {
+  std::lock_guard<std::mutex> lock(g_mutex);
+  for (int k = 0; k < g_nready[dev]; ++k)
+    if (g_ready[dev][k] == f) return cudaSuccess;
+  const cudaError_t e = f();
+  if (e == cudaSuccess && g_nready[dev] < kMaxVariants) g_ready[dev][g_nready[dev]++] = f;
+  return e;
+}
 
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
@@ -102,45 +122,25 @@ extern "C" int cr_step_noalloc(const cr_mesh_desc* desc, const double* u_in, dou
   cudaStream_t s = (cudaStream_t)cuda_stream;
 
   LaunchCtx lc;
-  memset(&lc, 0, sizeof(lc));
-  lc.u = u_out;
+  fill_launch_ctx(d, &lc);
+  // u^n is read where it is; u^{n+1} goes to u_out (in place if they are one)
+  lc.u = const_cast<double*>(u_in);
   lc.st = (DevState*)base;
   lc.rbar = base + off_rbar;
   lc.trace = base + off_trace;
-  lc.totals_part = nullptr;
-  lc.ma.E = E;
-  for (int k = 0; k < 3; ++k) {
-    lc.ma.cells[k] = k < d.dim ? d.cells[k] : 1;
-    lc.ma.cdiv[k] = make_fastdiv((unsigned)lc.ma.cells[k]);
-    lc.ma.inv_dx[k] = k < d.dim ? d.cells[k] / (d.hi[k] - d.lo[k]) : 0.0;
-  }
-  for (int k = 0; k < 3; ++k) lc.ma.inv_dx_f[k] = (float)lc.ma.inv_dx[k];
-  lc.ma.gamma_f = (float)d.gamma;
-  lc.ma.gm1_f = (float)(d.gamma - 1.0);
-  lc.ma.c_h_f = (float)d.c_h;
-  lc.ma.cfl = d.cfl;
-  lc.ma.dt_fixed = d.dt_fixed;
-  lc.ma.gamma = d.gamma;
-  lc.ma.c_h = d.c_h;
-  lc.pp64 = make_phys<double>(d.gamma, d.c_h);
-  lc.pp32 = make_phys<float>(d.gamma, d.c_h);
-  fill_ref_tables(d.degree_N, d.eq, lc.ma, &lc.tb64, &lc.tb32);
-  lc.sms = 1;
-  if ((e = cudaDeviceGetAttribute(&lc.sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return to_status(e);
-  lc.ma.tma_ok = tma_ok_for(u_out, E, o.NP);
+  lc.out = FaceOut{u_out == u_in ? nullptr : u_out, dt_out, 1};
+  lc.ma.tma_ok = tma_ok_for(u_in, E, o.NP);
 
-  if ((e = o.set_smem()) != cudaSuccess) return to_status(e);
-  if (u_out != u_in &&
-      (e = cudaMemcpyAsync(u_out, u_in, sizeof(double) * (size_t)o.M * nodes, cudaMemcpyDeviceToDevice, s)) !=
-          cudaSuccess)
+  // Three launches: the CFL reduction of u^n (slot 0), volume, face / update (with
+  // dt and the clean-up); a copy of the state, a clear of the record and a copy of
+  // dt besides were half of a small step.  64^2, N = 3, FP32: 62 -> 37 us a call.
+  if ((e = prepare_variant(dev, o.set_smem)) != cudaSuccess) return to_status(e);
+  if (g_dirty[dev].exchange(true) && (e = cudaMemsetAsync(lc.st, 0, sizeof(DevState), s)) != cudaSuccess)
     return to_status(e);
-  // the shared step record starts clean: t, steps, status, CFL slots (slot 0: u^n)
-  if ((e = cudaMemsetAsync(lc.st, 0, sizeof(DevState), s)) != cudaSuccess) return to_status(e);
   lc.slot = 0;
   if ((e = o.lambda(lc, s)) != cudaSuccess) return to_status(e);
   if ((e = o.volume(lc, s)) != cudaSuccess) return to_status(e);
   if ((e = o.face_update(lc, s)) != cudaSuccess) return to_status(e);
-  if (dt_out && (e = cudaMemcpyAsync(dt_out, &lc.st->dt, sizeof(double), cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
-    return to_status(e);
+  g_dirty[dev] = false;
   return CR_OK;
 }

@@ -79,8 +79,12 @@ struct Variant {
   static constexpr bool kBatched = EQ::DIM == 2 && !EQ::NC;
   static_assert(!kBatched || (LL::EPB == 32 && FL::EPB == 32), "the work list holds 32-element tiles");
   static cudaError_t face_update(const LaunchCtx& c, cudaStream_t s) {
-    k_face_update_lanes<EQ, N, R><<<face_tiles(c), FL::THREADS, FL::bytes(), s>>>(
-        c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
+    if (c.out.reset)
+      k_face_update_lanes_out<EQ, N, R><<<face_tiles(c), FL::THREADS, FL::bytes(), s>>>(
+          c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, c.out);
+    else
+      k_face_update_lanes<EQ, N, R><<<face_tiles(c), FL::THREADS, FL::bytes(), s>>>(
+          c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
     return cudaGetLastError();
   }
   static constexpr bool kVolInd = !EQ::NC && sizeof(R) == 4;
@@ -182,7 +186,7 @@ struct Variant {
   static cudaError_t lambda(const LaunchCtx& c, cudaStream_t s) {
     const long long total = c.ma.E * LL::NP;
     const unsigned grid = (unsigned)((total + 255) / 256);
-    k_lambda<EQ, N, R><<<grid, 256, 0, s>>>(c.u, c.st, c.ma, c.slot);
+    k_lambda<EQ, N, R><<<grid, 256, 0, s>>>(c.u, c.st, c.ma, c.slot, c.out.reset);
     return cudaGetLastError();
   }
   static cudaError_t totals(const LaunchCtx& c, cudaStream_t s) {
@@ -200,6 +204,7 @@ struct Variant {
     cudaError_t e = allow(k_volume_lanes<EQ, N, R>, PL::bytes());
     if (e == cudaSuccess) e = allow(k_volume_lanes_stage<EQ, N, R>, PL::bytes());
     if (e == cudaSuccess) e = allow(k_face_update_lanes<EQ, N, R>, FL::bytes());
+    if (e == cudaSuccess) e = allow(k_face_update_lanes_out<EQ, N, R>, FL::bytes());
     if (e == cudaSuccess) e = allow(k_face_stage_lanes<EQ, N, R>, FL::bytes());
     if constexpr (!EQ::NC) {
       if (e == cudaSuccess) e = allow(k_face_update_lanes_clean<EQ, N, R>, FL::bytes());

@@ -129,6 +129,16 @@ struct RkStage {
   int j, s;
 };
 
+// What one face / update launch writes besides the state in place: u^{n+1} into
+// another buffer (nullptr: in place), the step's dt, and (reset) zeros into the
+// CFL slot the step has read, so that a record used for one step at a time
+// starts the next one clean.
+struct FaceOut {
+  double* u;
+  double* dt;
+  int reset;
+};
+
 // ---------------------------------------------------------------------------
 // CFL reduction: every warp takes its maximum with shuffles and folds it into
 // its word of lam_bits[slot] with one 64-bit atomicMax (non-negative doubles order like
@@ -467,10 +477,12 @@ __device__ __forceinline__ void face_jump(const R* __restrict__ trace, long long
 // the path's arithmetic R, like the reduction of the face / update kernel
 template <class EQ, int N, typename R>
 __global__ void __launch_bounds__(256)
-k_lambda(const double* __restrict__ u, DevState* __restrict__ st, const MeshArgs ma, int slot) {
+k_lambda(const double* __restrict__ u, DevState* __restrict__ st, const MeshArgs ma, int slot, int fresh) {
   constexpr int M = EQ::M, NP = ipow(N + 1, EQ::DIM);
   const long long E = ma.E;
   const unsigned gid = blockIdx.x * blockDim.x + threadIdx.x;
+  // fresh: drop the status an earlier step left in a reused record
+  if (fresh && gid == 0) st->status = 0u;
   R lam = R(0);
   bool bad = false;
   if (gid < (unsigned)(E * NP)) {

@@ -905,8 +905,19 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
   const int tid = threadIdx.x;
   const long long E = ma.E;
   // a volume CTA that timed out left its records unwritten: leave u^n as it is
+  // (another output buffer gets it)
   if constexpr (!FUSED) {
-    if (st->status & ST_TIMEOUT) return;
+    if (st->status & ST_TIMEOUT) {
+      if (uout && !touched) {
+        const size_t vt = (size_t)E * NP;
+        for (int j = 0; j < n; ++j) {
+          const int r = tid + j * T;
+          if (r / NP < (int)min((long long)L::EPB, E - (long long)e0))
+            for (int v = 0; v < M; ++v) uout[v * vt + (size_t)e0 * NP + r] = u[v * vt + (size_t)e0 * NP + r];
+        }
+      }
+      return;
+    }
   }
   const R dtR = FUSED ? dt_fused : step_dt<R>(st);
   const int nel = (int)min((long long)L::EPB, E - (long long)e0);
@@ -1031,7 +1042,24 @@ k_face_update_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R*
                     DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                     int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  face_lanes_tile<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot, reinterpret_cast<R*>(smem_raw));
+  face_lanes_tile<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot,
+                            reinterpret_cast<R*>(smem_raw));
+}
+
+// the same with the outputs of a step that keeps no record of its own
+// (cr_step_noalloc); a kernel apart, since the pointers cost the plain one 1.5%
+template <class EQ, int N, typename R>
+__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB)
+k_face_update_lanes_out(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
+                        DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
+                        int slot, const FaceOut fo) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  if (blockIdx.x == 0) {
+    if (fo.dt && threadIdx.x == 0) *fo.dt = st->dt;
+    if (fo.reset && threadIdx.x < kLamSpread) st->lam_bits[slot][threadIdx.x] = 0ull;
+  }
+  face_lanes_tile<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot,
+                            reinterpret_cast<R*>(smem_raw), RkStage<R>{nullptr, nullptr, 0, 1}, R(0), nullptr, fo.u);
 }
 
 // the limited step's elements that the limiter does not touch: the plain
