@@ -18,7 +18,7 @@
 //   trace [DIM][2][NF][C][E] R   face data; side 0 = xi_d = 0 face, side 1 = xi_d = 1;
 //         per face node C components, each contiguous over the elements
 //         (a warp's 32 consecutive elements load one 128-byte line):
-//         U (M), F^d (M), lambda_d(u^n) (1) [+ GLM-MHD: F^nc,d (M), u^n (M)]
+//         U (M), F^d (M), lambda_d(u^n) (1) [+ GLM-MHD: u^n (M)]
 #pragma once
 #include "crkfr_async.cuh"
 #include "crkfr_physics.cuh"
@@ -213,7 +213,7 @@ __device__ __forceinline__ R step_dt(const DevState* st) {
 
 
 template <class EQ>
-__host__ __device__ constexpr int trace_comps() { return EQ::NC ? 4 * EQ::M + 1 : 2 * EQ::M + 1; }
+__host__ __device__ constexpr int trace_comps() { return EQ::NC ? 3 * EQ::M + 1 : 2 * EQ::M + 1; }
 // component c of the record of face node f of face (d, side) of element e
 template <class EQ, int NF>
 __host__ __device__ __forceinline__ size_t trace_index(int d, int side, int f, int c, long long E, long long e) {
@@ -411,7 +411,7 @@ __device__ __forceinline__ void load_face_record(const R* __restrict__ trace, lo
   for (int c = 0; c < C; ++c) rec[c] = ldx<COH>(p + (size_t)c * E);
 }
 
-// Jump J = F^num - F_own [+ B(u^n_own) g^avg(U) - F^nc_own] at one face node
+// Jump J = F^num - F_own [+ B(u^n_own) g^avg(U)] at one face node
 // from the own record o and the other side's record x (eq. numflux.cons and
 // the reduced-communication non-conservative flux of Sec. 2.3).
 template <class EQ, typename R>
@@ -424,20 +424,18 @@ __device__ __forceinline__ void jump_of(const R* o, const R* x, int d, int side_
   for (int v = 0; v < M; ++v)
     J[v] = mad(R(0.5), o[M + v] + x[M + v], mulr(R(-0.5) * lam * sgn, x[v] - o[v])) - o[M + v];
   if constexpr (EQ::NC) {
-    // + B(u^n_own) g^avg(U) - F^nc_own (the stage-wise flux adds its own sum
-    // in face_jump instead of the first term)
+    // + B(u^n_own) g^avg(U) (the stage-wise flux adds its own sum in face_jump
+    // instead); - F^nc_own is part of R-bar
     if constexpr (!EQ::NCS) {
       R un[M], q[EQ::P];
 #pragma unroll
-      for (int v = 0; v < M; ++v) un[v] = o[3 * M + 1 + v];
+      for (int v = 0; v < M; ++v) un[v] = o[2 * M + 1 + v];
       EQ::pair_data(un, q, pp);
       R g[2];
       g[0] = R(0.5) * (o[5 + d] + x[5 + d]);
       g[1] = R(0.5) * (o[8] + x[8]);
       EQ::nc_apply(d, q, g, J);
     }
-#pragma unroll
-    for (int v = 0; v < M; ++v) J[v] -= o[2 * M + 1 + v];
   }
 }
 
