@@ -34,22 +34,55 @@ struct Variant {
   using FL = FaceLaneLayout<EQ, N, R>;
   static_assert(PL::fits() && FL::fits(), "the lane layouts hold every variant");
   // resident CTAs per SM of the persistent volume kernel (computed once)
+  template <int SH>
   static int vol_occupancy() {
     static int occ = -1;
     if (occ < 0) {
+      using PS = PersistLayout<EQ, N, R, SH>;
       int nb = 0;
-      cudaFuncSetAttribute(k_volume_lanes<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PL::bytes());
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes<EQ, N, R>, LL::THREADS, PL::bytes());
+      cudaFuncSetAttribute(k_volume_lanes<EQ, N, R, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS::bytes());
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes<EQ, N, R, SH>, PS::L::THREADS, PS::bytes());
       occ = nb > 0 ? nb : 1;
     }
     return occ;
   }
-  static cudaError_t volume(const LaunchCtx& c, cudaStream_t s) {
-    const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;
-    const long long grid = std::min(ntiles, (long long)c.sms * vol_occupancy());
-    k_volume_lanes<EQ, N, R><<<(unsigned)grid, LL::THREADS, PL::bytes(), s>>>(
+  template <int SH>
+  static cudaError_t volume_shape(const LaunchCtx& c, cudaStream_t s) {
+    using PS = PersistLayout<EQ, N, R, SH>;
+    const long long ntiles = (c.ma.E + PS::L::EPB - 1) / PS::L::EPB;
+    const long long grid = std::min(ntiles, (long long)c.sms * vol_occupancy<SH>());
+    k_volume_lanes<EQ, N, R, SH><<<(unsigned)grid, PS::L::THREADS, PS::bytes(), s>>>(
         c.u, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
     return cudaGetLastError();
+  }
+  // FP64: tiles of 8 or 16 elements (LaneLayout<.., 2>).  The FP64 pipe bounds the
+  // launch, so its time is that of the SM with the most warps of work, and
+  // smaller tiles spread a mesh more evenly.  Where they fill whole warps (2D N = 1, 3,
+  // 5, 3D N = 1, 3) they are never more work and always taken; else where the
+  // busiest SM has fewer warps.  us per step, default against small tiles: 2D Euler N = 3
+  // 97x61 225 -> 171, 200^2 870 -> 850, N = 5 40x33 699 -> 505, 200^2 4492 -> 4265, GLM-MHD N = 3
+  // 97x61 596 -> 378, 61x45 310 -> 295, TGV N = 3 8x9x11 361 -> 238, 22x20x19 1297 -> 1270; by the
+  // rule: 2D N = 4 40x33 399 -> 324 (42 tiles, 5 warps against 3), 97x61 586 -> 548, but
+  // 200^2 2344 against 2659 (45 warps against 51), TGV N = 2 8x9x11 211 -> 116, 22x20x19
+  // 415 against 496.
+  static constexpr bool kSmall = sizeof(R) == 8 && EQ::DIM > 1 && LaneLayout<EQ, N, R, 2>::EPB < LL::EPB;
+  static constexpr bool kSmallOnly = kSmall && LaneLayout<EQ, N, R, 2>::THREADS % 32 == 0;
+  // warps of work on the SM with the most tiles
+  template <int SH>
+  static long long warps_per_sm(const LaunchCtx& c) {
+    using L = LaneLayout<EQ, N, R, SH>;
+    const long long ntiles = (c.ma.E + L::EPB - 1) / L::EPB;
+    return (ntiles + c.sms - 1) / c.sms * ((L::THREADS + 31) / 32);
+  }
+  static cudaError_t volume(const LaunchCtx& c, cudaStream_t s) {
+    if constexpr (kSmallOnly) {
+      return volume_shape<2>(c, s);
+    } else {
+      if constexpr (kSmall) {
+        if (warps_per_sm<2>(c) < warps_per_sm<0>(c)) return volume_shape<2>(c, s);
+      }
+      return volume_shape<0>(c, s);
+    }
   }
   static cudaError_t volume_stage(const LaunchCtx& c, cudaStream_t s, const double* u_in, int first) {
     const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;
@@ -201,7 +234,11 @@ struct Variant {
   }
   // dynamic shared memory of every kernel of the variant
   static cudaError_t set_smem() {
-    cudaError_t e = allow(k_volume_lanes<EQ, N, R>, PL::bytes());
+    cudaError_t e = cudaSuccess;
+    if constexpr (!kSmallOnly) e = allow(k_volume_lanes<EQ, N, R>, PL::bytes());
+    if constexpr (kSmall) {
+      if (e == cudaSuccess) e = allow(k_volume_lanes<EQ, N, R, 2>, PersistLayout<EQ, N, R, 2>::bytes());
+    }
     if (e == cudaSuccess) e = allow(k_volume_lanes_stage<EQ, N, R>, PL::bytes());
     if (e == cudaSuccess) e = allow(k_face_update_lanes<EQ, N, R>, FL::bytes());
     if (e == cudaSuccess) e = allow(k_face_update_lanes_out<EQ, N, R>, FL::bytes());
