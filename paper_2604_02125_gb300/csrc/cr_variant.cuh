@@ -2,6 +2,7 @@
 #pragma once
 #include "cr_internal.h"
 #include "crkfr_volume_lanes.cuh"
+#include "crkfr_volume_pairs.cuh"
 
 #include <algorithm>
 
@@ -75,6 +76,9 @@ struct Variant {
     return (ntiles + c.sms - 1) / c.sms * ((L::THREADS + 31) / 32);
   }
   static cudaError_t volume(const LaunchCtx& c, cudaStream_t s) {
+    if constexpr (kPairs) {
+      if (c.ma.E <= kPairElems * c.sms) return volume_pairs(c, s);
+    }
     if constexpr (kSmallOnly) {
       return volume_shape<2>(c, s);
     } else {
@@ -83,6 +87,18 @@ struct Variant {
       }
       return volume_shape<0>(c, s);
     }
+  }
+  // 1D, few elements: a lane per pair of nodes (k_volume_pairs).  The form with a
+  // thread per element takes the same time from 1 to 32 elements per SM; the
+  // pair form's grows beyond 8 to 16, and they meet at 35 to 80 elements per SM
+  // (FP32 with the Kennedy-Gruber flux, the cheapest, at 20 to 35).
+  static constexpr bool kPairs = EQ::DIM == 1 && !EQ::NC && EQ::VOL != VOL_CENTRAL && N >= 2;
+  static constexpr long long kPairElems = sizeof(R) == 4 && EQ::VOL == VOL_KEP ? 16 : 24;
+  static cudaError_t volume_pairs(const LaunchCtx& c, cudaStream_t s) {
+    constexpr int EPB = PairLanes<EQ, N>::EPB;
+    k_volume_pairs<EQ, N, R><<<(unsigned)((c.ma.E + EPB - 1) / EPB), 32, 0, s>>>(
+        c.u, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
+    return cudaGetLastError();
   }
   static cudaError_t volume_stage(const LaunchCtx& c, cudaStream_t s, const double* u_in, int first) {
     const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;

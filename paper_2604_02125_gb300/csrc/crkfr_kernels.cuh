@@ -308,8 +308,10 @@ __device__ __forceinline__ void line_differences(int d, const R (&q)[N + 1][EQ::
     const R c0 = R(2) * B[0][0], cN = R(2) * B[N][N];
 #pragma unroll
     for (int v = 0; v < M; ++v) {
-      acc[0][v] = c0 * fend[0][v];
-      acc[N][v] = cN * fend[1][v];
+      // 1D: rounded by itself, as in the form with a lane per pair (the sum of two
+      // products below would leave the fused one to the compiler)
+      acc[0][v] = EQ::DIM == 1 ? mulr(c0, fend[0][v]) : c0 * fend[0][v];
+      acc[N][v] = EQ::DIM == 1 ? mulr(cN, fend[1][v]) : cN * fend[1][v];
     }
 #pragma unroll
     for (int a = 0; a < n; ++a)

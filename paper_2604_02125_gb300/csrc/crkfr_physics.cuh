@@ -310,6 +310,16 @@ struct Euler {
   static constexpr bool NCS = false;   // stage-wise non-conservative flux (GLM-MHD only)
   static constexpr int IRHO = 0, IP = DIM_ + 1, IAUX = DIM_ + 2;
 
+  // A product that becomes pair data.  1D: rounded by itself, since a thread that
+  // holds a whole line would otherwise fuse it into the pairs' sums (v_a + v_b as
+  // u_a (1/rho_a) + v_b), which the form with a lane per pair cannot: both
+  // forms of the volume kernel take the same values.
+  template <typename R>
+  __device__ __forceinline__ static R value(R a, R b) {
+    if constexpr (DIM == 1) return mulr(a, b);
+    else return a * b;
+  }
+
   template <typename R>
   __device__ __forceinline__ static void pair_data(const R* u, R* q, const PhysParams<R>& pp) {
     R rho = u[0];
@@ -324,10 +334,10 @@ struct Euler {
       const R r = fast_rcp(prho * rho);
       const R ir = prho * r;                                         // 1 / rho
 #pragma unroll
-      for (int k = 0; k < DIM; ++k) q[1 + k] = u[1 + k] * ir;
+      for (int k = 0; k < DIM; ++k) q[1 + k] = value(u[1 + k], ir);
       q[0] = rho;
-      q[IP] = prho * ir;
-      q[IAUX] = rho * rho * rho * r;                                 // rho / p
+      q[IP] = value(prho, ir);
+      q[IAUX] = value(rho * rho * rho, r);                                 // rho / p
       return;
     }
     R ir = fast_rcp(rho);
@@ -335,14 +345,14 @@ struct Euler {
     q[0] = rho;
 #pragma unroll
     for (int k = 0; k < DIM; ++k) {
-      R v = u[1 + k] * ir;
+      R v = value(u[1 + k], ir);
       q[1 + k] = v;
       ke += v * u[1 + k];
     }
-    R p = (pp.gamma - R(1)) * (E - R(0.5) * ke);
+    R p = value(pp.gamma - R(1), E - R(0.5) * ke);
     q[IP] = p;
-    if constexpr (VOL == VOL_EC) q[IAUX] = rho * fast_rcp(p);
-    else q[IAUX] = E * ir;
+    if constexpr (VOL == VOL_EC) q[IAUX] = value(rho, fast_rcp(p));
+    else q[IAUX] = value(E, ir);
   }
 
   template <typename R>
@@ -353,7 +363,7 @@ struct Euler {
       for (int k = 0; k < DIM; ++k) ke += q[1 + k] * q[1 + k];
       return mad(q[IP], pp.inv_gm1, R(0.5) * q[0] * ke);
     }
-    return q[0] * q[IAUX];
+    return value(q[0], q[IAUX]);
   }
 
   // conserved variables from pair data

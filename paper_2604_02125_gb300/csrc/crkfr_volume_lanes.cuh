@@ -456,7 +456,7 @@ __device__ __forceinline__ void volume_lanes_tile(const double* __restrict__ u, 
           for (int v = 0; v < M; ++v) {
             const R r = ax[k][v] + (DIM > 1 ? my[L::O_RY + v * NP + l * n + k] : R(0));
             rb[k][v] += bp * r;
-            w[k][v] = ap * r;
+            w[k][v] = DIM == 1 ? mulr(ap, r) : ap * r;   // 1D: rounded as in k_volume_pairs
             if constexpr (rk_nsaved(N) > 0) ax[k][v] = r;
           }
         if constexpr (rk_nsaved(N) > 0) {

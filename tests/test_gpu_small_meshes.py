@@ -15,7 +15,8 @@ from parity_util import check_close
 pytestmark = pytest.mark.gpu
 
 # (system, dimension, cells of the small mesh, copies); 4864 = 32 x 152 elements in 2D and 3D
-MESHES = [("euler", 2, [16, 19], [4, 4]), ("euler", 3, [8, 8, 19], [2, 2, 1]),
+MESHES = [("euler", 1, [96], [512]), ("euler", 1, [77], [640]),
+          ("euler", 2, [16, 19], [4, 4]), ("euler", 3, [8, 8, 19], [2, 2, 1]),
           ("glm_mhd", 2, [16, 19], [4, 4])]
 
 
@@ -31,11 +32,13 @@ def _run(eq, dim, N, cells, vol, prec, U):
 
 
 @pytest.mark.parametrize("vol", ["ec", "kep", "central"])
-@pytest.mark.parametrize("prec", ["fp64"])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
 @pytest.mark.parametrize("eq,dim,cells,copies", MESHES)
 def test_copies(eq, dim, cells, copies, prec, vol):
     if eq == "glm_mhd" and vol == "kep":
         pytest.skip("no such flux")
+    if dim > 1 and prec == "fp32":
+        pytest.skip("one form")
     for N in range(1, 6):
         U, G, dt = _run(eq, dim, N, cells, vol, prec, None)
         tile = [1] + copies[::-1] + [1]
