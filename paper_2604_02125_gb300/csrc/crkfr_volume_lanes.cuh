@@ -873,8 +873,10 @@ struct FaceLaneLayout {
   // 1536 57.6 / 29.0 / 29.9 / 52 (spills); 64 batched solves 267 / 234 (1024) /
   // 221 (1152) / 228 (1280); RKFR 256^2 176 / 126 / 126 / 129.
   static constexpr int minb(int t) { return t / THREADS > 1 ? t / THREADS : 1; }
-  static constexpr int MINB = minb(sizeof(R) == 8 ? 512 : EQ::NC ? 768 : DIM == 3 ? 1536 : 1280), 
-                       MINB1 = minb(sizeof(R) == 8 ? 512 : EQ::NC ? 768 : 1152);
+  // 1D: 512, for the values loaded ahead.
+  static constexpr bool WIDE = sizeof(R) == 8 || DIM == 1;
+  static constexpr int MINB = minb(WIDE ? 512 : EQ::NC ? 768 : DIM == 3 ? 1536 : 1280),
+                       MINB1 = minb(WIDE ? 512 : EQ::NC ? 768 : 1152);
 };
 
 // One tile of EPB elements starting at e0 (sj: the CTA's shared memory; slot:
@@ -940,6 +942,25 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
   const size_t vs = (size_t)E * NP;   // values per variable
   const size_t g0 = (size_t)e0 * NP + tid;
 
+  // 1D: u^n and R-bar of all rounds ahead of phase A.  A round is M values a
+  // thread there, and a mesh of a few thousand elements has less than one warp
+  // per scheduler: each round's loads would be waited for in turn (us per step, FP32, before and
+  // after: 2046 elements N = 1 10.4 -> 9.5, N = 5 14.6 -> 12.5, 30000 elements N = 3 14.3 -> 13.3, N = 5 23.8 ->
+  // 22.8; 65536 N = 5 39.2 -> 37.4; FP64 within 1%, N = 1 20.1 -> 18.7).
+  constexpr int AHEAD = DIM == 1 ? n : 1;
+  double ua[AHEAD][M];
+  R ra[AHEAD][M];
+  if constexpr (DIM == 1) {
+#pragma unroll
+    for (int j = 0; j < n; ++j)
+      if ((tid + j * T) / NP < nel)
+#pragma unroll
+        for (int v = 0; v < M; ++v) {
+          ua[j][v] = u[g0 + j * T + v * vs];
+          ra[j][v] = ldx<FUSED>(rbar + g0 + j * T + v * vs);
+        }
+  }
+
   // ---- phase A: scaled jumps, -dt J^- g_R'(1)/dx at the xi = 1 faces and
   // +dt J^+ (-g_L'(0))/dx at the xi = 0 faces
   {
@@ -974,7 +995,7 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
   if constexpr (!F32) {
     if (last) thr = lambda_seen(st, FUSED ? slot : slot ^ 1);
   }
-#pragma unroll 1
+#pragma unroll AHEAD
   for (int j = 0; j < n; ++j) {
     const int r = tid + j * T, ee = r / NP, p = r % NP;
     const bool on = ee < nel && !(touched && touched[e0 + ee]);
@@ -984,8 +1005,13 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
       R du[M];
 #pragma unroll
       for (int v = 0; v < M; ++v) {
-        un[v] = u[g + v * vs];
-        du[v] = ldx<FUSED>(rbar + g + v * vs);
+        if constexpr (DIM == 1) {
+          un[v] = ua[j][v];
+          du[v] = ra[j][v];
+        } else {
+          un[v] = u[g + v * vs];
+          du[v] = ldx<FUSED>(rbar + g + v * vs);
+        }
       }
       // the jumps of the faces the node lies on (one at most per direction: one
       // addition, whichever side), then -dt R-bar
