@@ -29,7 +29,7 @@ Volume kernel (flux differencing, eq. entropy.cons.flux.dev, per stage):
 Face / update kernel (eq. numflux.cons, eq. crkfr.non.cons.final), bytes per
 DOF-update: u^n read and u^{n+1} written (FP64, 8M each), R-bar read (M in
 the path's arithmetic R), and the element's own face records, 2d faces x
-(NP/n) face nodes x C components x R per element, C = 2M+1 (GLM-MHD 4M+1);
+(NP/n) face nodes x C components x R per element, C = 2M+1 (GLM-MHD 3M+1);
 the neighbour's copy of a record is the same data, served by L2.
 """
 
@@ -78,7 +78,7 @@ def face_bytes(mesh, real_bytes):
     E = 1
     for k in range(d):
         E *= mesh["cells"][k]
-    C = 4 * M + 1 if mesh.get("eq", "euler") != "euler" else 2 * M + 1
+    C = 3 * M + 1 if mesh.get("eq", "euler") != "euler" else 2 * M + 1
     nodes = E * n ** d
     per_node = 8 * M + real_bytes * M + 8 * M + 2.0 * d * C * real_bytes / n
     return nodes * per_node
