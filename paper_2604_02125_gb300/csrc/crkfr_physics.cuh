@@ -295,6 +295,19 @@ struct MeshSpeeds {
   const float* inv_dx;
 };
 
+// Whether speed_bound's FP32 arithmetic held: density and its reciprocal, and every
+// 1/dx, normal numbers; the energy so large that the squares lost below the
+// normal range (1e-37) are within its error; the pressure above zero by more than
+// its error; the square of the speed (a2) of a size whose own square, which GLM-MHD
+// forms, is normal.  Too large a value makes up infinite or NaN.
+template <int DIM>
+__device__ __forceinline__ bool speed_range(float rho, float E, float p_low, float a2, float up, const MeshSpeeds& ms) {
+  bool ok = rho > 1e-30f && rho < 1e30f && E > 1e-28f && p_low > 1e-25f && a2 > 1e-17f && up < 1e38f;
+#pragma unroll
+  for (int k = 0; k < DIM; ++k) ok = ok && ms.inv_dx[k] >= 1.17549435e-38f;
+  return ok;
+}
+
 // ---------------------------------------------------------------------------
 // Compressible Euler in DIM dimensions: u = (rho, rho v_1..rho v_DIM, E).
 // Pair data q = (rho, v_1..v_DIM, p, aux); aux = rho/p for the EC flux,
@@ -449,21 +462,23 @@ struct Euler {
   // nothing).  With e = 2^-23: the inputs, the reciprocal and the roundings leave
   // |p - p_32| < 16 e (gamma - 1)(E + |m|^2/(2 rho)) and every other factor
   // within a few e; the bound takes p at its upper end and 32 e on the sum.
-  // Magnitudes whose FP32 parts could underflow are not certain.
+  // That holds while no part leaves the normal FP32 range by an amount that
+  // matters (speed_range): the kinetic energy is formed as m (m / rho), whose lost
+  // parts stay below 1e-37 against E > 1e-28, never from bare squares.
   __device__ __forceinline__ static bool speed_bound(const float* u, const MeshSpeeds& ms, float& up) {
     const float e16 = 16.0f / 8388608.0f;
     const float rho = u[0], Et = u[DIM + 1], ir = fast_rcp(rho);
     float ke = 0.0f;
 #pragma unroll
-    for (int k = 0; k < DIM; ++k) ke += u[1 + k] * u[1 + k];
-    const float kr = 0.5f * ke * ir, gm1 = ms.gm1;
+    for (int k = 0; k < DIM; ++k) ke += u[1 + k] * (u[1 + k] * ir);
+    const float kr = 0.5f * ke, gm1 = ms.gm1;
     const float p = gm1 * (Et - kr), dp = e16 * gm1 * (Et + kr);
-    const float c = speed_sqrt(ms.gamma * (p + dp) * ir);
+    const float c2 = ms.gamma * (p + dp) * ir, c = speed_sqrt(c2);
     float s = 0.0f;
 #pragma unroll
     for (int k = 0; k < DIM; ++k) s += (fabsf(u[1 + k]) * ir + c) * ms.inv_dx[k];
     up = s * (1.0f + 2.0f * e16);
-    return rho > 1e-30f && p - dp > 1e-25f && up < 1e38f;
+    return speed_range<DIM>(rho, Et, p - dp, c2, up, ms);
   }
 
   // physicality of a conserved state (rho > 0, p > 0, finite) and sum_d lambda_d / dx_d
@@ -637,7 +652,7 @@ struct GlmMhd {
     const float e16 = 16.0f / 8388608.0f;
     const float rho = u[0], ir = fast_rcp(rho), gm1 = ms.gm1;
     const float BB = u[5] * u[5] + u[6] * u[6] + u[7] * u[7];
-    const float q = 0.5f * ((u[1] * u[1] + u[2] * u[2] + u[3] * u[3]) * ir + BB + u[8] * u[8]);
+    const float q = 0.5f * (u[1] * (u[1] * ir) + u[2] * (u[2] * ir) + u[3] * (u[3] * ir) + BB + u[8] * u[8]);
     const float p = gm1 * (u[4] - q), dp = e16 * gm1 * (u[4] + q);
     const float a2 = ms.gamma * (p + dp) * ir, s = (a2 + BB * ir) * (1.0f + e16);
     float tot = 0.0f;
@@ -649,7 +664,7 @@ struct GlmMhd {
       tot += (fabsf(u[1 + d]) * ir + fmaxf(cf, ms.c_h)) * ms.inv_dx[d];
     }
     up = tot * (1.0f + 2.0f * e16);
-    return rho > 1e-30f && p - dp > 1e-25f && up < 1e38f;
+    return speed_range<2>(rho, u[4], p - dp, a2, up, ms);
   }
 
   template <typename T>
