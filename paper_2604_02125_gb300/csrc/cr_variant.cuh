@@ -125,9 +125,29 @@ struct Variant {
         c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, rk);
     return cudaGetLastError();
   }
+  // 1D: the update kernel with a thread per line (face_line) or per node
+  // (face_lanes_tile).  us per step, EC flux, line against node.  FP32: N = 1 9000
+  // elements 6.13 / 6.28, 131072 12.6 / 13.8; N = 3 9000 9.10 / 9.47, 131072 21.5 /
+  // 23.0, 262144 33.6 / 35.3: always the line.  N = 2 64 5.73 / 5.97, 16000 7.31 /
+  // 7.43; its lines of three have no 16-byte accesses, and from the
+  // L2's capacity on a thread per node moves them better (262144 26.1 / 24.8).  N = 4 and 5 hold too much
+  // per thread: N = 4 64 8.71 / 8.47, 30000 16.5 / 15.8, 262144 (face launch) 24.5 /
+  // 18.9.  FP64, all degrees: N = 5 64 41.9 / 43.9, 2046 52.1 / 52.8; N = 4 30000
+  // (face launch) 19.9 / 18.6, 65536 32.6 / 27.8.
+  static bool face_by_line(const LaunchCtx& c) {
+    if (sizeof(R) == 8) return c.ma.E <= 96LL * c.sms;
+    return N == 1 || N == 3 || (N == 2 && c.ma.E <= 1024LL * c.sms);
+  }
   static constexpr bool kBatched = EQ::DIM == 2 && !EQ::NC;
   static_assert(!kBatched || (LL::EPB == 32 && FL::EPB == 32), "the work list holds 32-element tiles");
   static cudaError_t face_update(const LaunchCtx& c, cudaStream_t s) {
+    if constexpr (EQ::DIM == 1) {
+      if (!c.out.reset && face_by_line(c)) {
+        k_face_update_line<EQ, N, R><<<face_tiles(c), FL::THREADS, 0, s>>>(
+            c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot);
+        return cudaGetLastError();
+      }
+    }
     if (c.out.reset)
       k_face_update_lanes_out<EQ, N, R><<<face_tiles(c), FL::THREADS, FL::bytes(), s>>>(
           c.u, (const R*)c.rbar, (const R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, c.out);

@@ -873,10 +873,11 @@ struct FaceLaneLayout {
   // 1536 57.6 / 29.0 / 29.9 / 52 (spills); 64 batched solves 267 / 234 (1024) /
   // 221 (1152) / 228 (1280); RKFR 256^2 176 / 126 / 126 / 129.
   static constexpr int minb(int t) { return t / THREADS > 1 ? t / THREADS : 1; }
-  // 1D: 512, for the values loaded ahead.
+  // 1D: 512, for the values loaded ahead; none for the form with a thread per line.
   static constexpr bool WIDE = sizeof(R) == 8 || DIM == 1;
   static constexpr int MINB = minb(WIDE ? 512 : EQ::NC ? 768 : DIM == 3 ? 1536 : 1280),
-                       MINB1 = minb(WIDE ? 512 : EQ::NC ? 768 : 1152);
+                       MINB1 = DIM == 1 ? 1 : minb(WIDE ? 512 : EQ::NC ? 768 : 1152),
+                       MINB_OUT = DIM == 1 ? 1 : MINB;
 };
 
 // One tile of EPB elements starting at e0 (sj: the CTA's shared memory; slot:
@@ -1078,6 +1079,167 @@ __device__ __forceinline__ void face_lanes_tile(double* __restrict__ u, const R*
   if (last) reduce_lambda<R>(lam, bad, st, FUSED ? slot : slot ^ 1);
 }
 
+// n contiguous values of one line, in 16-byte accesses where VEC says that lines start
+// on such a boundary (an array that does and an even n, or four floats, give it)
+template <int n, bool VEC, typename T>
+__device__ __forceinline__ void load_line(const T* __restrict__ src, T (&out)[n]) {
+  constexpr int W = 16 / (int)sizeof(T);
+  if constexpr (VEC && n % W == 0) {
+#pragma unroll
+    for (int k = 0; k < n / W; ++k) {
+      const uint4 x = reinterpret_cast<const uint4*>(src)[k];
+      memcpy(&out[k * W], &x, 16);
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < n; ++k) out[k] = src[k];
+  }
+}
+template <int n, bool VEC, typename T>
+__device__ __forceinline__ void store_line(T* __restrict__ dst, const T (&in)[n]) {
+  constexpr int W = 16 / (int)sizeof(T);
+  if constexpr (VEC && n % W == 0) {
+#pragma unroll
+    for (int k = 0; k < n / W; ++k) {
+      uint4 x;
+      memcpy(&x, &in[k * W], 16);
+      reinterpret_cast<uint4*>(dst)[k] = x;
+    }
+  } else {
+#pragma unroll
+    for (int k = 0; k < n; ++k) dst[k] = in[k];
+  }
+}
+
+// 1D: a thread per element (its line of n nodes), the jumps of its two faces in
+// registers, no exchange and no barrier.  The face part of a small mesh is one
+// round trip to memory, which the two phases of face_lanes_tile make two, and an
+// RKFR stage is a chain of them: the earlier increments K_q come in one load of
+// all of a line's values per q here, not one per round and q.  Arithmetic and
+// order are face_lanes_tile's: the same bits.  us per step, EC flux, two phases ->
+// here: RKFR FP32 N = 3 64 elements 27.9 -> 20.6, 262144 130 -> 100, N = 5 64 77.5 -> 48.5, 9000
+// 83.7 -> 60.0, 262144 545 -> 357, FP64 N = 5 2046 247 -> 224; limited FP32 N = 3 64 14.0 -> 11.3;
+// the single-stage update's figures are at Variant::face_by_line.
+// VEC: u and the output start on 16-byte boundaries (this library's own arrays do).
+template <class EQ, int N, typename R, bool RK = false, bool VEC = true>
+__device__ __forceinline__ void face_line(double* __restrict__ u, const R* __restrict__ rbar,
+                                          const R* __restrict__ trace, DevState* __restrict__ st, const MeshArgs& ma,
+                                          const PhysParams<R>& pp, const RefTab<R>& tb, int slot,
+                                          const RkStage<R>& rk = RkStage<R>{nullptr, nullptr, 0, 1},
+                                          const unsigned char* __restrict__ touched = nullptr,
+                                          double* __restrict__ uout = nullptr) {
+  static_assert(EQ::DIM == 1, "one line per element");
+  constexpr int M = EQ::M, n = N + 1;
+  constexpr bool F32 = sizeof(R) == 4;
+  const long long E = ma.E;
+  const unsigned e = blockIdx.x * blockDim.x + threadIdx.x;
+  const size_t vs = (size_t)E * n, g = (size_t)e * n;
+  bool on = (long long)e < E;
+  // as face_lanes_tile: u^n stays, another output buffer gets it
+  if (st->status & ST_TIMEOUT) {
+    if (uout && !touched && on)
+      for (int v = 0; v < M; ++v)
+        for (int k = 0; k < n; ++k) uout[v * vs + g + k] = u[v * vs + g + k];
+    return;
+  }
+  on = on && !(touched && touched[e]);
+  const bool last = !RK || rk.j == rk.s - 1;   // uniform over the grid
+  double* dst = uout ? uout : u;
+  if (RK && !last) dst = rk.uout;
+  const R dtR = step_dt<R>(st);
+  double un[M][n];
+  if (on) {
+    R du[M][n];
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+      load_line<n, true>(rbar + v * vs + g, du[v]);
+      load_line<n, VEC>(u + v * vs + g, un[v]);
+    }
+    const unsigned ec[3] = {e, 0, 0};
+    R J[2][M];
+#pragma unroll
+    for (int side = 1; side >= 0; --side) {
+      face_jump<EQ, N, R>(trace, E, 0, side, e, neighbour_of(e, ec, 0, side ? +1 : -1, ma), 0, J[side], pp, tb);
+      const R sc = side ? -(dtR * tb.iwN * inv_dx_of<R>(ma, 0)) : dtR * tb.iw0 * inv_dx_of<R>(ma, 0);
+#pragma unroll
+      for (int v = 0; v < M; ++v) J[side][v] = mulr(sc, J[side][v]);
+    }
+#pragma unroll
+    for (int v = 0; v < M; ++v)
+#pragma unroll
+      for (int k = 0; k < n; ++k) du[v][k] = mad(-dtR, du[v][k], k == 0 ? J[0][v] : k == N ? J[1][v] : R(0));
+    if constexpr (RK) {
+      const R cj = last ? tb.b[rk.j] : tb.a[rk.j + 1][rk.j];
+      R acc[M][n];
+#pragma unroll
+      for (int v = 0; v < M; ++v) {
+        if (!last) store_line<n, true>(rk.k + (size_t)rk.j * M * vs + v * vs + g, du[v]);
+#pragma unroll
+        for (int k = 0; k < n; ++k) acc[v][k] = mulr(cj, du[v][k]);
+      }
+#pragma unroll 1
+      for (int q = 0; q < rk.j; ++q) {
+        const R c = last ? tb.b[q] : tb.a[rk.j + 1][q];
+        if (c != R(0)) {
+#pragma unroll
+          for (int v = 0; v < M; ++v) {
+            R kq[n];
+            load_line<n, true>(rk.k + (size_t)q * M * vs + v * vs + g, kq);
+#pragma unroll
+            for (int k = 0; k < n; ++k) acc[v][k] = mad(c, kq[k], acc[v][k]);
+          }
+        }
+      }
+#pragma unroll
+      for (int v = 0; v < M; ++v)
+#pragma unroll
+        for (int k = 0; k < n; ++k) du[v][k] = acc[v][k];
+    }
+#pragma unroll
+    for (int v = 0; v < M; ++v) {
+#pragma unroll
+      for (int k = 0; k < n; ++k) {
+        if constexpr (F32) un[v][k] += f2d_int(du[v][k]);
+        else un[v][k] += du[v][k];
+      }
+    }
+  }
+  // the reduction's atomics are under way when the stores begin
+  if (last) {
+    R lam = R(0);
+    bool bad = false;
+    float thr = 0.0f;
+    if constexpr (!F32) thr = lambda_seen(st, slot ^ 1);
+#pragma unroll
+    for (int k = 0; k < n; ++k) {
+      double uu[M];
+#pragma unroll
+      for (int v = 0; v < M; ++v) uu[v] = un[v][k];
+      if constexpr (F32) {
+        if (on) {
+          R lk;
+          bad = bad || !physical_state<EQ, R>(uu, ma, lk);
+          lam = fmax(lam, lk);
+        }
+      } else {
+        wave_speeds_fp64<EQ>(on, uu, ma, thr, lam, bad);
+      }
+    }
+    reduce_lambda<R>(lam, bad, st, slot ^ 1);
+  }
+  if (on) {
+#pragma unroll
+    for (int v = 0; v < M; ++v) store_line<n, VEC>(dst + v * vs + g, un[v]);
+  }
+}
+
+template <class EQ, int N, typename R>
+__global__ void __launch_bounds__(32)
+k_face_update_line(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
+                   DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb, int slot) {
+  face_line<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, slot);
+}
+
 template <class EQ, int N, typename R>
 __global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB)
 k_face_update_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
@@ -1091,7 +1253,7 @@ k_face_update_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R*
 // the same with the outputs of a step that keeps no record of its own
 // (cr_step_noalloc); a kernel apart, since the pointers cost the plain one 1.5%
 template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB)
+__global__ void __launch_bounds__(FaceLaneLayout<EQ, N, R>::THREADS, FaceLaneLayout<EQ, N, R>::MINB_OUT)
 k_face_update_lanes_out(double* __restrict__ u, const R* __restrict__ rbar, const R* __restrict__ trace,
                         DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                         int slot, const FaceOut fo) {
@@ -1100,8 +1262,18 @@ k_face_update_lanes_out(double* __restrict__ u, const R* __restrict__ rbar, cons
     if (fo.dt && threadIdx.x == 0) *fo.dt = st->dt;
     if (fo.reset && threadIdx.x < kLamSpread) st->lam_bits[slot][threadIdx.x] = 0ull;
   }
-  face_lanes_tile<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot,
-                            reinterpret_cast<R*>(smem_raw), RkStage<R>{nullptr, nullptr, 0, 1}, R(0), nullptr, fo.u);
+  if constexpr (EQ::DIM == 1) {
+    // the caller's arrays: any 8-byte boundary
+    const RkStage<R> none{nullptr, nullptr, 0, 1};
+    if (((reinterpret_cast<size_t>(u) | reinterpret_cast<size_t>(fo.u)) & 15) == 0)
+      face_line<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, slot, none, nullptr, fo.u);
+    else
+      face_line<EQ, N, R, false, false>(u, rbar, trace, st, ma, pp, tb, slot, none, nullptr, fo.u);
+  } else {
+    face_lanes_tile<EQ, N, R>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB,
+                              slot, reinterpret_cast<R*>(smem_raw), RkStage<R>{nullptr, nullptr, 0, 1}, R(0), nullptr,
+                              fo.u);
+  }
 }
 
 // the limited step's elements that the limiter does not touch: the plain
@@ -1113,8 +1285,12 @@ k_face_update_lanes_clean(double* __restrict__ uin, double* __restrict__ uout, c
                           DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                           int slot) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  face_lanes_tile<EQ, N, R>(uin, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot, reinterpret_cast<R*>(smem_raw),
-                            RkStage<R>{nullptr, nullptr, 0, 1}, R(0), touched, uout);
+  if constexpr (EQ::DIM == 1)
+    face_line<EQ, N, R>(uin, rbar, trace, st, ma, pp, tb, slot, RkStage<R>{nullptr, nullptr, 0, 1}, touched, uout);
+  else
+    face_lanes_tile<EQ, N, R>(uin, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB,
+                              slot, reinterpret_cast<R*>(smem_raw), RkStage<R>{nullptr, nullptr, 0, 1}, R(0), touched,
+                              uout);
 }
 
 // face / update part of stage rk.j of the multi-stage RKFR step
@@ -1124,8 +1300,12 @@ k_face_stage_lanes(double* __restrict__ u, const R* __restrict__ rbar, const R* 
                    DevState* __restrict__ st, const MeshArgs ma, const PhysParams<R> pp, const RefTab<R> tb,
                    int slot, const RkStage<R> rk) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  face_lanes_tile<EQ, N, R, true>(u, rbar, trace, st, ma, pp, tb, blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot,
-                                  reinterpret_cast<R*>(smem_raw), rk);
+  if constexpr (EQ::DIM == 1)
+    face_line<EQ, N, R, true>(u, rbar, trace, st, ma, pp, tb, slot, rk);
+  else
+    face_lanes_tile<EQ, N, R, true>(u, rbar, trace, st, ma, pp, tb,
+                                    blockIdx.x * (unsigned)FaceLaneLayout<EQ, N, R>::EPB, slot,
+                                    reinterpret_cast<R*>(smem_raw), rk);
 }
 
 // ---------------------------------------------------------------------------
