@@ -871,12 +871,14 @@ struct FaceLaneLayout {
   // 1024 / 1280 / 1536: 2D Euler 256^2 N = 3 29.8 / 23.0 / 21.0 / 22.7, TGV
   // 64^3 N = 3 797 / 559 / 556 / 513; GLM-MHD 128^2 N = 4 none / 768 / 1024 /
   // 1536 57.6 / 29.0 / 29.9 / 52 (spills); 64 batched solves 267 / 234 (1024) /
-  // 221 (1152) / 228 (1280); RKFR 256^2 176 / 126 / 126 / 129.
+  // 221 (1152) / 228 (1280); RKFR 256^2 176 / 126 / 126 / 129.  3D N = 1, whose jumps
+  // are most of its work, spills at 1536: 1024 (22x20x19 14.3 -> 10.5, 48^3 69.8 -> 53.5;
+  // 768 56.4, 1280 54.6; the limited step's 15.7 -> 14.9, RKFR 32^3 31.0 -> 30.6).
   static constexpr int minb(int t) { return t / THREADS > 1 ? t / THREADS : 1; }
   // 1D: 512, for the values loaded ahead; none for the form with a thread per line.
   static constexpr bool WIDE = sizeof(R) == 8 || DIM == 1;
-  static constexpr int MINB = minb(WIDE ? 512 : EQ::NC ? 768 : DIM == 3 ? 1536 : 1280),
-                       MINB1 = DIM == 1 ? 1 : minb(WIDE ? 512 : EQ::NC ? 768 : 1152),
+  static constexpr int MINB = minb(WIDE ? 512 : EQ::NC ? 768 : DIM == 3 ? (N == 1 ? 1024 : 1536) : 1280),
+                       MINB1 = DIM == 1 ? 1 : minb(WIDE ? 512 : EQ::NC ? 768 : DIM == 3 && N == 1 ? 1024 : 1152),
                        MINB_OUT = DIM == 1 ? 1 : MINB;
 };
 
