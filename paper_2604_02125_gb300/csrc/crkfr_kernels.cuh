@@ -426,16 +426,17 @@ __device__ __forceinline__ void jump_of(const R* o, const R* x, int d, int side_
   for (int v = 0; v < M; ++v)
     J[v] = mad(R(0.5), o[M + v] + x[M + v], mulr(R(-0.5) * lam * sgn, x[v] - o[v])) - o[M + v];
   if constexpr (EQ::NC) {
-    // + B(u^n_own) g^avg(U) (the stage-wise flux adds its own sum in face_jump
-    // instead); - F^nc_own is part of R-bar
+    // + B(u^n_own) (g^avg(U) - g(u^n_own)) (the stage-wise flux adds its own sum in
+    // face_jump instead); the rest of - F^nc_own is part of R-bar
+    // (nonconservative_ends)
     if constexpr (!EQ::NCS) {
       R un[M], q[EQ::P];
 #pragma unroll
       for (int v = 0; v < M; ++v) un[v] = o[2 * M + 1 + v];
       EQ::pair_data(un, q, pp);
       R g[2];
-      g[0] = R(0.5) * (o[5 + d] + x[5 + d]);
-      g[1] = R(0.5) * (o[8] + x[8]);
+      g[0] = R(0.5) * ((o[5 + d] - un[5 + d]) + (x[5 + d] - un[5 + d]));
+      g[1] = R(0.5) * ((o[8] - un[8]) + (x[8] - un[8]));
       EQ::nc_apply(d, q, g, J);
     }
   }
@@ -450,7 +451,8 @@ __device__ __forceinline__ void face_jump(const R* __restrict__ trace, long long
   load_face_record<EQ, N, R, COH>(trace, E, d, 1 - side_own, f, e_oth, x);
   jump_of<EQ, R>(o, x, d, side_own, J, pp);
   if constexpr (EQ::NCS) {
-    // + sum_j b_j B(u^(j)_own) g^avg(u^(j)) (eq. bad.numflux.non.cons)
+    // + sum_j b_j B(u^(j)_own) (g^avg - g)(u^(j)), F^nc_own of eq.
+    // bad.numflux.non.cons included
 #pragma unroll 1
     for (int j = 0; j < rk_stages(N); ++j) {
       R wo[7], wx[7];
@@ -462,8 +464,8 @@ __device__ __forceinline__ void face_jump(const R* __restrict__ trace, long long
       R go[2], gx[2], g[2], nc[EQ::M];
       EQ::ncg_prims(d, wo, go);
       EQ::ncg_prims(d, wx, gx);
-      g[0] = R(0.5) * (go[0] + gx[0]);
-      g[1] = R(0.5) * (go[1] + gx[1]);
+      g[0] = R(0.5) * (gx[0] - go[0]);
+      g[1] = R(0.5) * (gx[1] - go[1]);
 #pragma unroll
       for (int v = 0; v < EQ::M; ++v) nc[v] = R(0);
       EQ::nc_apply_prims(d, wo, g, nc);
