@@ -126,6 +126,29 @@ bool get_ops(int eq, int dim, int prec, int vol, int N, VariantOps* o, int ncflu
   return false;
 }
 
+// The rows of D add up to zero (a uniform flux has no residual); rounded after
+// the scaling by 1/dx they miss it by an ulp of their largest entry, which a
+// large uniform pressure turns into the leading error.  The diagonal of the
+// end rows, the smallest off-diagonal entry of an inner row (whose diagonal
+// is zero), is taken as minus the sum of the others, rounded once.
+template <typename R>
+static void close_row(int N, int p, const double (&D)[6][6], R (&row)[6]) {
+  int m = p;
+  if (p > 0 && p < N) {
+    for (int q = 0; q <= N; ++q)
+      if (q != p && (m == p || std::fabs(D[p][q]) < std::fabs(D[p][m]))) m = q;
+    row[p] = R(0);
+  }
+  double hi = 0.0, lo = 0.0;   // the sum and what its additions lost (Knuth's two-sum)
+  for (int q = 0; q <= N; ++q) {
+    if (q == m) continue;
+    const double x = row[q], t = hi + x, bb = t - hi;
+    lo += (hi - (t - bb)) + (x - bb);
+    hi = t;
+  }
+  row[m] = (R)-(hi + lo);
+}
+
 void fill_ref_tables(int N, int eq, const MeshArgs& ma, RefTab<double>* t64, RefTab<float>* t32) {
   // nodes, weights and D of the degree: computed on first use (Newton's method)
   struct Ref {
@@ -141,33 +164,21 @@ void fill_ref_tables(int N, int eq, const MeshArgs& ma, RefTab<double>* t64, Ref
   std::memset(t64, 0, sizeof(*t64));
   std::memset(t32, 0, sizeof(*t32));
   const double sa = eq == CR_EULER ? 2.0 : 0.5;   // row scale of the two-point flux (RefTab::A)
-  for (int d = 0; d < 4; ++d)
+  for (int d = 0; d < 4; ++d) {
+    const double sc = d < 3 ? ma.inv_dx[d] : 1.0;
     for (int p = 0; p <= N; ++p) {
-      const double sc = d < 3 ? ma.inv_dx[d] : 1.0;
       for (int q = 0; q <= N; ++q) {
         t64->B[d][p][q] = D[p][q] * sc;
         t32->B[d][p][q] = (float)t64->B[d][p][q];
       }
-      // The rows of D add up to zero (a uniform flux has no residual); rounded
-      // to FP32 they miss it by an ulp of their largest entry, which a large
-      // uniform pressure turns into the form's leading error.  The diagonal of
-      // the end rows, the smallest off-diagonal entry of an inner row (whose
-      // diagonal is zero), is taken as minus the sum of the others.
-      int m = p;
-      if (p > 0 && p < N) {
-        for (int q = 0; q <= N; ++q)
-          if (q != p && (m == p || std::fabs(D[p][q]) < std::fabs(D[p][m]))) m = q;
-        t32->B[d][p][p] = 0.0f;
-      }
-      double rest = 0.0;
-      for (int q = 0; q <= N; ++q)
-        if (q != m) rest += (double)t32->B[d][p][q];
-      t32->B[d][p][m] = (float)-rest;
+      close_row(N, p, D, t64->B[d][p]);
+      close_row(N, p, D, t32->B[d][p]);
       for (int q = 0; q <= N; ++q) {
         t64->A[d][p][q] = sa * t64->B[d][p][q];
         t32->A[d][p][q] = (float)sa * t32->B[d][p][q];
       }
     }
+  }
   for (int p = 0; p < 6; ++p) {
     for (int q = 0; q < 6; ++q) {
       t32->A2[0][p][q] = make_float2(t32->A[0][p][q], t32->A[1][p][q]);
