@@ -179,11 +179,13 @@ __device__ __forceinline__ double unit_plus(float uh, float ul, float c1h, float
   const float oh = __fadd_rn(c1h, nh), ol = __fadd_rn(nh, -__fadd_rn(oh, -c1h)) + c1l + nl;
   const float ch = __fmul_rn(uh, oh), cl = __fmaf_rn(uh, oh, -ch) + __fmaf_rn(uh, ol, ul * oh);
   const float magic = 12582912.0f;   // 1.5 2^23
-  const float x = __fmaf_rn(ch, 2147483648.0f, magic);                       // ch in steps of 2^-31
-  const float rem = __fmaf_rn(-__fadd_rn(x, -magic), 4.656612873077393e-10f, ch) + cl;
+  // ch in steps of 2^-34 (at most 2^21.4 of them): the rest, below 2^-35, keeps its bits to 2^-59 when
+  // cl joins it.  In steps of 2^-31 that sum was rounded at 2^-57, close to the final 2^-54.
+  const float x = __fmaf_rn(ch, 17179869184.0f, magic);
+  const float rem = __fmaf_rn(-__fadd_rn(x, -magic), 5.820766091346741e-11f, ch) + cl;
   const float y = __fmaf_rn(rem, NEG ? 9007199254740992.0f : 4503599627370496.0f, magic);
   const int ih = __float_as_int(x) - 0x4B400000, il = __float_as_int(y) - 0x4B400000;
-  const long long i = (long long)ih * (1ll << (NEG ? 22 : 21)) + il + ((long long)unit << 32);
+  const long long i = (long long)ih * (1ll << (NEG ? 19 : 18)) + il + ((long long)unit << 32);
   return __longlong_as_double(i);
 }
 
@@ -208,9 +210,9 @@ static __device__ __noinline__ void logmean_pair_far(double a1, double b1, doubl
 // 1 is a correction below 2^-12.6, two FP32 parts give it to 2^-57, and integer
 // arithmetic adds it to 1.  Nine FP64 instructions a pair (four sums, a
 // three-FMA reciprocal, two products) against 22 with the polynomials in FP64;
-// the result's error is that of its roundings, as there (against 128 bits, for
-// u < 2^-11: 1/F within 9.9e-17 and F within 1.5e-16, root mean square 3.3e-17 and
-// 6.4e-17; FP64 Horner 3.2e-17 and 6.4e-17).  Volume launch: 256^2, N = 3 1558 -> 1227
+// the result's error is that of its one rounding, as there (against 113 bits, for
+// u < 1e-4: root mean square 3.2e-17 for 1/F and 6.4e-17 for F, FP64 Horner 3.2e-17 and 6.4e-17;
+// L 7.4e-17 either way, 1/L 1.04e-16 against 1.23e-16 with the reciprocal of a product).  Volume launch: 256^2, N = 3 1558 -> 1227
 // us, 97x61 N = 5 1266 -> 951, 64-element 1D wave 64 -> 53, GLM-MHD 128^2 N = 4 3267 ->
 // 2933.  Above 2^-11 (a/b > 1.045) the degree-8
 // polynomials in FP64, above 1/16 the logarithms (a single FP64 series bound at
