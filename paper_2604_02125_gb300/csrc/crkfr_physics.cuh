@@ -75,14 +75,29 @@ template <> struct LogMeanEps<float> { static constexpr float v = 0.05f; };
 
 // FP64: the reciprocal unit's approximation r of 1/x (relative error about
 // 2^-20) and one third-order Householder iteration, r (1 + e + e^2) with
-// e = 1 - x r: three FP64 fused multiply-adds, error e^3 plus one rounding.
+// e = 1 - x r: three FP64 fused multiply-adds, error e^3 plus one rounding.  The
+// unit takes subnormal operands and results for zero, so this holds for 2^-1022 <=
+// |x| < 2^1022 (rcp_normal); fast_rcp scales the others into that range and back, and
+// leaves zero and the infinities (e is NaN) to the unit.
 // FP32: the MUFU reciprocal (rcp.approx, about 1 ulp), no slow-path branch.
-__device__ __forceinline__ double fast_rcp(double x) {
+__device__ __forceinline__ double rcp_unit(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  const double e = fma(-x, r, 1.0);
+  return r;
+}
+__device__ __forceinline__ double rcp_normal(double x) {
+  const double r = rcp_unit(x), e = fma(-x, r, 1.0);
   return fma(r, fma(e, e, e), r);
 }
+__device__ __forceinline__ bool rcp_holds(double x) {
+  return (((unsigned)__double2hiint(x) >> 20) & 0x7FFu) - 1u < 2044u;
+}
+__device__ __forceinline__ double rcp_scaled(double x) {
+  const double sc = fabs(x) < 1.0 ? 1.2676506002282294e30 : 7.8886090522101181e-31;   // 2^100, 2^-100
+  const double y = x * sc, r = rcp_unit(y), e = fma(-y, r, 1.0);
+  return e == e ? fma(r, fma(e, e, e), r) * sc : r;
+}
+__device__ __forceinline__ double fast_rcp(double x) { return rcp_holds(x) ? rcp_normal(x) : rcp_scaled(x); }
 __device__ __forceinline__ float fast_rcp(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -143,7 +158,8 @@ __device__ __forceinline__ void logmean_pair(float a1, float b1, float a2, float
 
 // u = (d/s)^2 as the sum of two FP32 values (relative error about 2^-45), from the
 // bits of d and s: both are scaled by the power of two that takes s to [1, 2).
-// False where that fails: s not a normal number, or |d| >= 2 |s| (or not finite).
+// False where that fails: |d| >= 2 |s| (or not finite), |s| below 2^-895, where the
+// exponent of d = 0 would not be small beside that of s, or |s| beyond rcp_normal's range.
 __device__ __forceinline__ bool ratio_squared(double d, double s, float& uh, float& ul) {
   const unsigned sH = (unsigned)__double2hiint(s), sL = (unsigned)__double2loint(s);
   const unsigned dH = (unsigned)__double2hiint(d), dL = (unsigned)__double2loint(d);
@@ -162,7 +178,7 @@ __device__ __forceinline__ bool ratio_squared(double d, double s, float& uh, flo
   q1 = __fmaf_rn(__fmaf_rn(-q1, sh, rem), r, q1);
   uh = __fmul_rn(q0, q0);
   ul = __fmaf_rn(q0 + q0, q1, __fmaf_rn(q0, q0, -uh));
-  return (unsigned)(es - 1) < 2046u && k <= 0;
+  return (unsigned)(es - 128) < 1917u && k <= 0;
 }
 
 // 1 + u (c1 + u (c2 + u (c3 + u (c4 + u c5)))) for 0 <= u < 2^-11 as a double,
@@ -221,7 +237,7 @@ static __device__ __noinline__ void logmean_pair_far(double a1, double b1, doubl
 __device__ __forceinline__ void logmean_pair(double a1, double b1, double a2, double b2, double& H1, double& T2,
                                              double& rs2) {
   const double s1 = a1 + b1, d1 = a1 - b1, s2 = a2 + b2, d2 = a2 - b2;
-  rs2 = fast_rcp(s2);
+  rs2 = rcp_normal(s2);
   float h1, l1, h2, l2;
   const bool ok1 = ratio_squared(d1, s1, h1, l1), ok2 = ratio_squared(d2, s2, h2, l2);
   if (ok1 && ok2 && fmaxf(h1, h2) < 4.8828125e-4f) {   // 2^-11
@@ -231,6 +247,7 @@ __device__ __forceinline__ void logmean_pair(double a1, double b1, double a2, do
     T2 = rs2 * unit_plus<false>(h2, l2, 0.33333334f, -9.9341078e-9f, 0.2f, -2.9802323e-9f, 1.0f / 7.0f, 1.0f / 9.0f,
                                 1.0f / 11.0f, 0x3FF00000u);
   } else {
+    if (!rcp_holds(s2)) rs2 = rcp_scaled(s2);
     logmean_pair_far(a1, b1, a2, b2, rs2, H1, T2);
   }
 }

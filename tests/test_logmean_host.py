@@ -100,3 +100,18 @@ def test_two_part_series_is_rounded_once(host, fmax):
         e_inv, e_F = _series(u)
         assert abs(4 * Fraction(iF4[k]) - e_inv) <= Fraction(1, 2 ** 54) + Fraction(1, 2 ** 59), (k, float(u))
         assert abs(Fraction(F[k]) - e_F) <= Fraction(1, 2 ** 53) + Fraction(1, 2 ** 59), (k, float(u))
+
+
+@pytest.mark.parametrize("e", [-1021, -1017, -1000, -897, -896, -895, -894, 1020, 1021, 1022])
+def test_sums_at_the_ends_of_the_range(host, e):
+    """Equal and nearly equal values whose sum 2^(e+1) lies at either end of the FP64
+    range, where the exponent field of a zero difference is not small beside the
+    sum's and the reciprocal unit takes operands or results for zero.  Two roundings, and
+    the subnormal result's own beyond 2^1022."""
+    s = np.full(3, 2.0 ** e)
+    d = s * np.array([0.0, 2.0 ** -20, -2.0 ** -12]) if e > -900 else np.zeros(3)
+    iF4, F = _call(host.units, d, s)
+    for k in range(3):
+        e_inv, e_F = _series((Fraction(d[k]) / Fraction(s[k])) ** 2)
+        assert abs(4 * Fraction(iF4[k]) - e_inv) <= Fraction(1, 2 ** 52), (e, k, iF4[k])
+        assert abs(Fraction(F[k]) - e_F) <= Fraction(1, 2 ** 50), (e, k, F[k])
