@@ -15,8 +15,9 @@
 // contents, so calls that overlap on the GPU (on different streams, or from
 // several threads) race; the step record is clean at the start of every
 // call (the face kernel zeroes the CFL slot its step has read, the first
-// kernel the status; a call whose launches failed makes the next one clear
-// it whole).  The array's device address is looked up on the first call on each
+// kernel drops a timeout; a call whose launches failed makes the next one clear
+// it whole).  Its non-physical bit, which this entry point does not report, stays
+// once it is set.  The array's device address is looked up on the first call on each
 // device and kept for the life of the process; cudaDeviceReset destroys the
 // context that address belongs to, so a process that resets a device must
 // not call this entry point on that device afterwards.

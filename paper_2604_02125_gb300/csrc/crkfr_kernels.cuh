@@ -483,8 +483,10 @@ k_lambda(const double* __restrict__ u, DevState* __restrict__ st, const MeshArgs
   constexpr int M = EQ::M, NP = ipow(N + 1, EQ::DIM);
   const long long E = ma.E;
   const unsigned gid = blockIdx.x * blockDim.x + threadIdx.x;
-  // fresh: drop the status an earlier step left in a reused record
-  if (fresh && gid == 0) st->status = 0u;
+  // fresh: drop the timeout an earlier step left in a reused record.  Only that bit,
+  // which nothing in this launch sets: a store of 0 could fall on either side of
+  // the other warps' atomicOr of ST_NONPHYS.
+  if (fresh && gid == 0) atomicAnd(&st->status, ~ST_TIMEOUT);
   R lam = R(0);
   bool bad = false;
   if (gid < (unsigned)(E * NP)) {
