@@ -5,6 +5,7 @@
 #include "crkfr_volume_pairs.cuh"
 
 #include <algorithm>
+#include <atomic>
 
 namespace crk {
 
@@ -28,24 +29,36 @@ template <> struct PPB<float> {
   static const RefTab<float>& tab(const BatchLaunch& b) { return b.tb32; }
 };
 
+constexpr int kOccDevices = 64;   // devices whose occupancies are kept
+
 template <class EQ, int N, typename R>
 struct Variant {
   using LL = LaneLayout<EQ, N, R>;
   using PL = PersistLayout<EQ, N, R>;
   using FL = FaceLaneLayout<EQ, N, R>;
   static_assert(PL::fits() && FL::fits(), "the lane layouts hold every variant");
-  // resident CTAs per SM of the persistent volume kernel (computed once)
+  // Resident CTAs per SM of a persistent kernel on the current device, whose
+  // shared-memory allowance set_smem has raised: asked for once per device (a call
+  // costs several microseconds), by whichever thread comes first, since
+  // all of them get the same answer.  0: not known yet.
+  using OccCache = std::atomic<int>[kOccDevices];
+  template <class K>
+  static int occupancy_of(OccCache& cache, K k, int threads, size_t bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) dev = -1;
+    const bool known = dev >= 0 && dev < kOccDevices;
+    int nb = known ? cache[dev].load(std::memory_order_relaxed) : 0;
+    if (nb == 0) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k, threads, bytes);
+      if (known) cache[dev].store(nb, std::memory_order_relaxed);
+    }
+    return nb;
+  }
   template <int SH>
   static int vol_occupancy() {
-    static int occ = -1;
-    if (occ < 0) {
-      using PS = PersistLayout<EQ, N, R, SH>;
-      int nb = 0;
-      cudaFuncSetAttribute(k_volume_lanes<EQ, N, R, SH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PS::bytes());
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes<EQ, N, R, SH>, PS::L::THREADS, PS::bytes());
-      occ = nb > 0 ? nb : 1;
-    }
-    return occ;
+    using PS = PersistLayout<EQ, N, R, SH>;
+    static OccCache occ;
+    return std::max(1, occupancy_of(occ, k_volume_lanes<EQ, N, R, SH>, PS::L::THREADS, PS::bytes()));
   }
   template <int SH>
   static cudaError_t volume_shape(const LaunchCtx& c, cudaStream_t s) {
@@ -108,15 +121,8 @@ struct Variant {
     return cudaGetLastError();
   }
   static int vol_stage_occupancy() {
-    static int occ = -1;
-    if (occ < 0) {
-      int nb = 0;
-      cudaFuncSetAttribute(k_volume_lanes_stage<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)PL::bytes());
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes_stage<EQ, N, R>, LL::THREADS, PL::bytes());
-      occ = nb > 0 ? nb : 1;
-    }
-    return occ;
+    static OccCache occ;
+    return std::max(1, occupancy_of(occ, k_volume_lanes_stage<EQ, N, R>, LL::THREADS, PL::bytes()));
   }
   static unsigned face_tiles(const LaunchCtx& c) { return (unsigned)((c.ma.E + FL::EPB - 1) / FL::EPB); }
   static cudaError_t face_stage(const LaunchCtx& c, cudaStream_t s, int j, int ns) {
@@ -159,16 +165,10 @@ struct Variant {
   static constexpr bool kVolInd = !EQ::NC && sizeof(R) == 4;
   static cudaError_t volume_ind(const LaunchCtx& c, cudaStream_t s) {
     if constexpr (kVolInd) {
-      static int occ = -1;
-      if (occ < 0) {
-        int nb = 0;
-        cudaFuncSetAttribute(k_volume_lanes_ind<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)PL::bytes());
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_volume_lanes_ind<EQ, N, R>, LL::THREADS, PL::bytes());
-        occ = nb > 0 ? nb : 1;
-      }
+      static OccCache occ;
+      const int per_sm = std::max(1, occupancy_of(occ, k_volume_lanes_ind<EQ, N, R>, LL::THREADS, PL::bytes()));
       const long long ntiles = (c.ma.E + LL::EPB - 1) / LL::EPB;
-      const long long grid = std::min(ntiles, (long long)c.sms * occ);
+      const long long grid = std::min(ntiles, (long long)c.sms * per_sm);
       k_volume_lanes_ind<EQ, N, R><<<(unsigned)grid, LL::THREADS, PL::bytes(), s>>>(
           c.u, (R*)c.rbar, (R*)c.trace, c.st, c.ma, PP<R>::get(c), PP<R>::tab(c), c.slot, c.araw, c.tcount, c.lt);
       return cudaGetLastError();
@@ -219,16 +219,11 @@ struct Variant {
   using FU = FusedLayout<EQ, N, R>;
   static constexpr bool kFused = FU::fits() && !EQ::NC && LL::EPB == 32;
   static int fused_occupancy() {
-    static int occ = -1;
-    if (occ < 0) {
-      int nb = 0;
-      if constexpr (kFused) {
-        cudaFuncSetAttribute(k_step_fused<EQ, N, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FU::bytes());
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_fused<EQ, N, R>, LL::THREADS, FU::bytes());
-      }
-      occ = nb;
+    if constexpr (kFused) {
+      static OccCache occ;
+      return occupancy_of(occ, k_step_fused<EQ, N, R>, LL::THREADS, FU::bytes());
     }
-    return occ;
+    return 0;
   }
   static cudaError_t step_fused(const LaunchCtx& c, cudaStream_t s, int phase) {
     if constexpr (kFused) {
@@ -276,6 +271,9 @@ struct Variant {
       if (e == cudaSuccess) e = allow(k_volume_lanes<EQ, N, R, 2>, PersistLayout<EQ, N, R, 2>::bytes());
     }
     if (e == cudaSuccess) e = allow(k_volume_lanes_stage<EQ, N, R>, PL::bytes());
+    if constexpr (kVolInd) {
+      if (e == cudaSuccess) e = allow(k_volume_lanes_ind<EQ, N, R>, PL::bytes());
+    }
     if (e == cudaSuccess) e = allow(k_face_update_lanes<EQ, N, R>, FL::bytes());
     if (e == cudaSuccess) e = allow(k_face_update_lanes_out<EQ, N, R>, FL::bytes());
     if (e == cudaSuccess) e = allow(k_face_stage_lanes<EQ, N, R>, FL::bytes());
