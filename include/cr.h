@@ -266,9 +266,11 @@ int cr_step_noalloc(const cr_mesh_desc *desc, const double *u_in, double *u_out,
  * context without the limiter.  Synchronises the stream. */
 int cr_get_blend_alpha(cr_ctx *ctx, double *alpha, int on_device);
 
-/* JSON description of the kernel configuration chosen for the context (the
- * autotuned persistent grids of the batched form), copied into buf (len
- * bytes, NUL-terminated).  CR_EINVAL if it does not fit. */
+/* JSON description of the kernel configuration chosen for the context, copied
+ * into buf (len bytes, NUL-terminated): the autotuned persistent grids of the
+ * batched form; for a single solve "scheme", "step" (split or fused), "volume"
+ * (lanes, small tiles or pairs) with its "elements_per_cta", and "face" (lanes,
+ * line or limited per-node).  CR_EINVAL if it does not fit. */
 int cr_tuning_info(cr_ctx *ctx, char *buf, size_t len);
 
 /* Release every device buffer and graph of the context. */

@@ -890,12 +890,21 @@ int cr_tuning_info(cr_ctx* c, char* buf, size_t len) {
   if (c->batched) {
     info = batched_tuning(c->batched);
   } else {
+    // the forms the step launches (launch_step): the RKFR stages, the limited FP32
+    // step and the single launch have the lane form of the volume kernel only, and
+    // in 1D the stages and the limited step the face kernel with a thread per line
+    const VariantOps& o = c->ops;
+    const bool rk = c->desc[0].scheme == CR_SCHEME_RKFR;
+    const VolForm vf = rk || c->fused || (c->limited && o.volume_ind) ? VolForm::Lanes : o.vol_form(c->lc);
+    const char* vol = vf == VolForm::Pairs ? "pairs" : vf == VolForm::SmallTiles ? "small tiles" : "lanes";
+    const int elems = vf == VolForm::Pairs ? o.pair_elems : vf == VolForm::SmallTiles ? o.small_elems : o.lane_elems;
+    const bool line = !c->fused && o.dim == 1 && (rk || c->limited || o.face_by_line(c->lc));
     char tmp[256];
     std::snprintf(tmp, sizeof(tmp),
                   "{\"scheme\": \"%s\", \"step\": \"%s\", \"volume\": \"%s\", \"elements_per_cta\": %d, "
                   "\"face\": \"%s\"}",
-                  c->desc[0].scheme == CR_SCHEME_RKFR ? "rkfr" : "crkfr", c->fused ? "fused" : "split",
-                  "lanes", c->ops.lane_elems, c->limited ? "limited per-node" : "lanes");
+                  rk ? "rkfr" : "crkfr", c->fused ? "fused" : "split", vol, elems,
+                  c->limited ? "limited per-node" : line ? "line" : "lanes");
     info = tmp;
   }
   std::snprintf(buf, len, "%s", info.c_str());

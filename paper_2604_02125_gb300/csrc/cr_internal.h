@@ -55,10 +55,15 @@ struct BatchLaunch {
   int shape;          // volume kernel shape (0: default, 1: alternative; chosen by the autotuner)
 };
 
+// the kernel a single-stage step's volume part runs (Variant::vol_form)
+enum class VolForm { Lanes, SmallTiles, Pairs };
+
 struct VariantOps {
   int M, NP, NF, C, dim;       // C: components of a face record
   size_t ncs_per_elem;         // stage-wise non-conservative flux: stage-trace values per element after the records
-  int lane_elems;              // elements per CTA of the volume kernel
+  VolForm (*vol_form)(const LaunchCtx&);                 // of the single-stage step's volume kernel, for this mesh
+  int lane_elems, small_elems, pair_elems;               // elements per CTA of VolForm's kernels
+  bool (*face_by_line)(const LaunchCtx&);                // of the single-stage step's face / update kernel
   size_t real_bytes;           // sizeof(R)
   cudaError_t (*volume)(const LaunchCtx&, cudaStream_t);
   cudaError_t (*face_update)(const LaunchCtx&, cudaStream_t);

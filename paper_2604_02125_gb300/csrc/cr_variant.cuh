@@ -88,18 +88,27 @@ struct Variant {
     const long long ntiles = (c.ma.E + L::EPB - 1) / L::EPB;
     return (ntiles + c.sms - 1) / c.sms * ((L::THREADS + 31) / 32);
   }
-  static cudaError_t volume(const LaunchCtx& c, cudaStream_t s) {
+  // the form for a mesh: decides the launch and what cr_tuning_info reports
+  static VolForm vol_form(const LaunchCtx& c) {
     if constexpr (kPairs) {
-      if (c.ma.E <= kPairElems * c.sms) return volume_pairs(c, s);
+      if (c.ma.E <= kPairElems * c.sms) return VolForm::Pairs;
     }
-    if constexpr (kSmallOnly) {
-      return volume_shape<2>(c, s);
-    } else {
-      if constexpr (kSmall) {
-        if (warps_per_sm<2>(c) < warps_per_sm<0>(c)) return volume_shape<2>(c, s);
-      }
-      return volume_shape<0>(c, s);
+    if constexpr (kSmallOnly) return VolForm::SmallTiles;
+    if constexpr (kSmall) {
+      if (warps_per_sm<2>(c) < warps_per_sm<0>(c)) return VolForm::SmallTiles;
     }
+    return VolForm::Lanes;
+  }
+  static cudaError_t volume(const LaunchCtx& c, cudaStream_t s) {
+    const VolForm form = vol_form(c);
+    if constexpr (kPairs) {
+      if (form == VolForm::Pairs) return volume_pairs(c, s);
+    }
+    if constexpr (kSmall) {
+      if (kSmallOnly || form == VolForm::SmallTiles) return volume_shape<2>(c, s);
+    }
+    if constexpr (!kSmallOnly) return volume_shape<0>(c, s);
+    return cudaErrorNotSupported;
   }
   // 1D, few elements: a lane per pair of nodes (k_volume_pairs).  The form with a
   // thread per element takes the same time from 1 to 32 elements per SM; the
@@ -141,6 +150,7 @@ struct Variant {
   // 18.9.  FP64, all degrees: N = 5 64 41.9 / 43.9, 2046 52.1 / 52.8; N = 4 30000
   // (face launch) 19.9 / 18.6, 65536 32.6 / 27.8.
   static bool face_by_line(const LaunchCtx& c) {
+    if (EQ::DIM > 1) return false;
     if (sizeof(R) == 8) return c.ma.E <= 96LL * c.sms;
     return N == 1 || N == 3 || (N == 2 && c.ma.E <= 1024LL * c.sms);
   }
@@ -336,7 +346,12 @@ struct Variant {
     o->C = trace_comps<EQ>();
     o->ncs_per_elem = EQ::NCS ? ncs_values_per_elem<EQ, N>() : 0;
     o->dim = EQ::DIM;
+    o->vol_form = &vol_form;
     o->lane_elems = LL::EPB;
+    o->small_elems = LaneLayout<EQ, N, R, 2>::EPB;
+    if constexpr (kPairs) o->pair_elems = PairLanes<EQ, N>::EPB;
+    else o->pair_elems = 0;
+    o->face_by_line = &face_by_line;
     o->real_bytes = sizeof(R);
     o->volume = &volume;
     o->face_update = &face_update;
