@@ -313,11 +313,6 @@ struct cr_ctx {
   // in ubuf[p] (the limited step reads one and writes the other)
   double* ubuf[2] = {nullptr, nullptr};
   bool limited = false;
-  // limiter, FP32 form: the indicator kernels run on a second stream beside
-  // the volume kernel (both only read u^n; the indicator uses the FP64 pipe,
-  // the volume kernel the FP32 one), joined before the face kernels
-  cudaStream_t side = nullptr;
-  cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
   // device buffers carved out of a caller's workspace (cr_init_mesh_ws): not freed here
   bool borrowed = false;
   cudaStream_t cap_stream = nullptr;
@@ -381,11 +376,6 @@ static void free_single(cr_ctx* c) {
     c->g1[p] = c->g16[p] = nullptr;
   }
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
-  if (c->side) cudaStreamDestroy(c->side);
-  if (c->ev_fork) cudaEventDestroy(c->ev_fork);
-  if (c->ev_join) cudaEventDestroy(c->ev_join);
-  c->side = nullptr;
-  c->ev_fork = c->ev_join = nullptr;
   if (!c->borrowed) {
     cudaFree(c->ubuf[0]);
     cudaFree(c->ubuf[1]);
@@ -435,21 +425,13 @@ static int launch_step(cr_ctx* c, cudaStream_t s, int parity) {
     c->lc.u = state_buf(c, parity);
     c->lc.u_next = state_buf(c, parity ^ 1);
     if (c->ops.volume_ind) {
-      // FP32 lane form: the volume kernel evaluates the raw coefficients of
-      // the tiles it has finished, then the smoothing pass
+      // FP32: the volume kernel evaluates the raw coefficients of the tiles it
+      // has finished, then the smoothing pass
       CR_TRY(c->ops.volume_ind(c->lc, s));
       CR_TRY(c->ops.alpha_smooth(c->lc, s));
-    } else if (c->desc[0].prec == CR_FP32_PAIRFLUX) {
-      // FP32 form: the FP64 indicator beside the FP32 volume kernel
-      // (measured 0.164 -> 0.155 ms per step at 256^2, N = 3)
-      CR_TRY(cudaEventRecord(c->ev_fork, s));
-      CR_TRY(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
-      CR_TRY(c->ops.alpha(c->lc, c->side));
-      CR_TRY(cudaEventRecord(c->ev_join, c->side));
-      CR_TRY(c->ops.volume(c->lc, s));
-      CR_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
     } else {
-      // FP64 form: both would compete for the FP64 pipe (measured slower side by side)
+      // FP64: the indicator and the volume kernel compete for the FP64 pipe
+      // (measured slower side by side)
       CR_TRY(c->ops.alpha(c->lc, s));
       CR_TRY(c->ops.volume(c->lc, s));
     }
@@ -508,7 +490,7 @@ static int plan_single(cr_ctx* c, std::vector<BufSpec>* plan) {
   // one partial sum per CTA of the totals kernel (256 nodes per CTA)
   c->totals_blocks = (size_t)((nodes + 255) / 256);
   c->limited = d.limiter == CR_LIMITER_BLENDING;
-  if (c->limited && (!o.alpha || !o.face_limited)) return CR_EINVAL;
+  if (c->limited && !o.face_limited) return CR_EINVAL;
   // the single-launch step (crkfr_fused.cuh) on request only:
   // CRKFR_STEP_KERNELS=fused in the environment, for variants that have one.
   // Measured slower than the two kernels on every workload (the face / update
@@ -582,9 +564,6 @@ static int init_single(cr_ctx* c, void* workspace = nullptr) {
   if (e == cudaSuccess && c->fused) e = cudaMemsetAsync(lc.flags, 0, sizeof(unsigned) * (size_t)((E + 31) / 32), c->stream);
   if (e != cudaSuccess) { free_single(c); return cuda_status(e); }
   e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
-  if (e == cudaSuccess && c->limited) e = cudaStreamCreateWithFlags(&c->side, cudaStreamNonBlocking);
-  if (e == cudaSuccess && c->limited) e = cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming);
-  if (e == cudaSuccess && c->limited) e = cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming);
   if (e != cudaSuccess) { free_single(c); return cuda_status(e); }
   for (int p = 0; p < c->nphase && rc == CR_OK; ++p) {
     rc = capture(c, 1, p, &c->g1[p]);

@@ -186,20 +186,20 @@ struct Variant {
     return cudaErrorNotSupported;
   }
   static cudaError_t alpha_smooth(const LaunchCtx& c, cudaStream_t s) {
-    if constexpr (!EQ::NC) {
-      if constexpr (kVolInd)
-        k_alpha_fix<EQ, N><<<(unsigned)((c.ma.E + 127) / 128), 128, 0, s>>>(c.u, c.araw, c.ma, c.lt);
+    if constexpr (kVolInd) {
+      k_alpha_fix<EQ, N><<<(unsigned)((c.ma.E + 127) / 128), 128, 0, s>>>(c.u, c.araw, c.ma, c.lt);
       k_alpha_smooth<EQ::DIM><<<(unsigned)((c.ma.E + 255) / 256), 256, 0, s>>>(c.araw, c.alpha, c.touched, c.tlist,
                                                                               c.tcount, c.ma);
       return cudaGetLastError();
     }
     return cudaErrorNotSupported;
   }
+  // FP64: the raw coefficients, then the smoothing pass (FP32: volume_ind, alpha_smooth)
   static cudaError_t alpha(const LaunchCtx& c, cudaStream_t s) {
-    if constexpr (!EQ::NC) {
-      constexpr int T = AlphaRawLayout<EQ, N, R>::THREADS;
+    if constexpr (!EQ::NC && !kVolInd) {
+      constexpr int T = AlphaRawLayout<EQ, N>::THREADS;
       const unsigned grid = (unsigned)((c.ma.E + T - 1) / T);
-      k_alpha_raw<EQ, N, R><<<grid, T, 0, s>>>(c.u, c.araw, c.tcount, c.ma, c.lt);
+      k_alpha_raw<EQ, N><<<grid, T, 0, s>>>(c.u, c.araw, c.tcount, c.ma, c.lt);
       k_alpha_smooth<EQ::DIM><<<(unsigned)((c.ma.E + 255) / 256), 256, 0, s>>>(c.araw, c.alpha, c.touched, c.tlist,
                                                                               c.tcount, c.ma);
       return cudaGetLastError();
@@ -359,10 +359,10 @@ struct Variant {
     o->face_stage = &face_stage;
     o->lambda = &lambda;
     o->step_fused = kFused ? &step_fused : nullptr;
-    o->alpha = EQ::NC ? nullptr : &alpha;
+    o->alpha = EQ::NC || kVolInd ? nullptr : &alpha;
     o->face_limited = EQ::NC ? nullptr : &face_limited;
     o->volume_ind = kVolInd ? &volume_ind : nullptr;
-    o->alpha_smooth = EQ::NC ? nullptr : &alpha_smooth;
+    o->alpha_smooth = kVolInd ? &alpha_smooth : nullptr;
     o->totals = &totals;
     o->set_smem = &set_smem;
   }

@@ -5,9 +5,9 @@
 //  k_alpha_raw           per element: the modal smoothness indicator of rho p
 //                        (energy fraction of the highest orthonormal Legendre
 //                        modes), the logistic map, its clips and the cap
-//                        alpha_max; FP64, or in the FP32 form FP32 with the
-//                        FP64 evaluation near the clip thresholds.  One thread
-//                        per element.
+//                        alpha_max, in FP64.  One thread per element.  FP32
+//                        form: in the volume kernel (k_volume_lanes_ind), with the
+//                        FP64 evaluation near the clip thresholds (k_alpha_fix).
 //  k_alpha_smooth        per element: a_e = max(raw_e, raw_nb / 2 over the
 //                        face neighbours), and whether the limiter touches
 //                        the element (a_e or a face neighbour's a above zero,
@@ -35,8 +35,6 @@
 // first-order fluxes read neighbouring nodes of other elements), so a limited
 // context ping-pongs between two buffers.
 #pragma once
-#include <type_traits>
-
 #include "crkfr_kernels.cuh"
 
 namespace crk {
@@ -117,34 +115,24 @@ __device__ __forceinline__ T indicator_of_values(Load load, const LimTab& lt) {
   return En;
 }
 
-// Energy fraction of the highest modes of one element's rho p (see
-// k_alpha_raw).  FP64: E = max((T - T1)/T, (T1 - T2)/T1) from the three sums;
-// FP32: the top and second-top energies summed directly (sums of squares, no
-// cancellation), E = max(Ttop/T, Tsec/(T - Ttop)).
-template <class EQ, int N, typename T>
-__device__ __forceinline__ T indicator_energy(const double* __restrict__ u, long long E, long long e,
-                                              const MeshArgs& ma, const LimTab& lt) {
+// Energy fraction of the highest modes of one element's rho p in FP64 (see
+// k_alpha_raw): E = max((T - T1)/T, (T1 - T2)/T1) from the three sums.  (FP32: the top and
+// second-top energies summed directly, sums of squares without cancellation, E = max(Ttop/T,
+// Tsec/(T - Ttop)).)
+template <class EQ, int N>
+__device__ __forceinline__ double indicator_energy(const double* __restrict__ u, long long E, long long e,
+                                                   const MeshArgs& ma, const LimTab& lt) {
   constexpr int DIM = EQ::DIM, NP = ipow(N + 1, DIM);
-  constexpr bool F32 = sizeof(T) == 4;
-  return indicator_of_values<EQ, N, T>([&](int p) {
-    T rho, Et, mm = T(0);
-    if constexpr (F32) {
-      rho = d2f_int(u[(size_t)e * NP + p]);
-      Et = d2f_int(u[((size_t)(DIM + 1) * E + e) * NP + p]);
-    } else {
-      rho = u[(size_t)e * NP + p];
-      Et = u[((size_t)(DIM + 1) * E + e) * NP + p];
-    }
+  return indicator_of_values<EQ, N, double>([&](int p) {
+    const double rho = u[(size_t)e * NP + p], Et = u[((size_t)(DIM + 1) * E + e) * NP + p];
+    double mm = 0.0;
 #pragma unroll
     for (int k = 0; k < DIM; ++k) {
-      T mk;
-      if constexpr (F32) mk = d2f_int(u[((size_t)(1 + k) * E + e) * NP + p]);
-      else mk = u[((size_t)(1 + k) * E + e) * NP + p];
+      const double mk = u[((size_t)(1 + k) * E + e) * NP + p];
       mm += mk * mk;
     }
     // rho p = (gamma - 1)(rho E - |m|^2 / 2)
-    const T gm1 = F32 ? T(ma.gamma_f - 1.0f) : T(ma.gamma - 1.0);
-    return gm1 * (rho * Et - T(0.5) * mm);
+    return (ma.gamma - 1.0) * (rho * Et - 0.5 * mm);
   }, lt);
 }
 
@@ -163,7 +151,7 @@ __device__ __forceinline__ float alpha_of_energy_f32(float En, const LimTab& lt)
 template <class EQ, int N>
 __device__ __forceinline__ double alpha_raw_fp64(const double* __restrict__ u, long long E, long long e,
                                               const MeshArgs& ma, const LimTab& lt) {
-  const double En = indicator_energy<EQ, N, double>(u, E, e, ma, lt);
+  const double En = indicator_energy<EQ, N>(u, E, e, ma, lt);
   double a = 1.0 / (1.0 + exp(-(lt.sharp / lt.tau) * (En - lt.tau)));
   if (a < 0.001) a = 0.0;
   if (a > 0.999) a = 1.0;
@@ -182,81 +170,60 @@ k_alpha_fix(const double* __restrict__ u, double* __restrict__ araw, const MeshA
 // Elements per block of k_alpha_raw (one thread each) when their rho p values
 // fit the static shared memory (48 KB), else 0: every thread reads its own
 // element's values from global memory.
-template <class EQ, int N, typename R>
+template <class EQ, int N>
 struct AlphaRawLayout {
-  using T = typename std::conditional<sizeof(R) == 4, float, double>::type;
   static constexpr int NP = ipow(N + 1, EQ::DIM);
-  static constexpr int FIT = 49152 / (int)((NP + 1) * sizeof(T)) / 32 * 32;
+  static constexpr int FIT = 49152 / (int)((NP + 1) * sizeof(double)) / 32 * 32;
   static constexpr int EB = FIT >= 128 ? 128 : FIT >= 32 ? FIT : 0;
   static constexpr int THREADS = EB > 0 ? EB : 128;
 };
 
 // ---------------------------------------------------------------------------
-// Blending coefficient per element before smoothing.  The FP64 form evaluates
-// it in FP64 throughout.  The FP32 form evaluates the energy fraction in FP32
-// and takes the FP64 evaluation for the elements whose FP32 value lies within
-// 2% of a clip threshold, so every clip decision is the FP64 one (the FP32
-// value's relative error is below 1e-4 there); elsewhere the logistic map in
-// FP32 differs from the FP64 one by about 1e-6.
+// Blending coefficient per element before smoothing, FP64 form.  (The FP32 form
+// evaluates the energy fraction in FP32 in its volume kernel, k_volume_lanes_ind, and takes
+// the FP64 evaluation, k_alpha_fix, for the elements whose FP32 value lies within
+// 2% of a clip threshold, so every clip decision is the FP64 one -- the FP32
+// value's relative error is below 1e-4 there; elsewhere the logistic map in
+// FP32 differs from the FP64 one by about 1e-6.)
 // ---------------------------------------------------------------------------
-template <class EQ, int N, typename R>
-__global__ void __launch_bounds__(AlphaRawLayout<EQ, N, R>::THREADS)
+template <class EQ, int N>
+__global__ void __launch_bounds__(AlphaRawLayout<EQ, N>::THREADS)
 k_alpha_raw(const double* __restrict__ u, double* __restrict__ araw, unsigned* __restrict__ tcount, const MeshArgs ma,
             const LimTab lt) {
-  constexpr int DIM = EQ::DIM, NP = ipow(N + 1, DIM), EB = AlphaRawLayout<EQ, N, R>::EB;
-  using T = typename AlphaRawLayout<EQ, N, R>::T;
+  constexpr int DIM = EQ::DIM, NP = ipow(N + 1, DIM), EB = AlphaRawLayout<EQ, N>::EB;
   const long long E = ma.E;
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   // the touched list of this step starts empty (k_alpha_smooth fills it after
   // this kernel; the last step's limited kernel has read it before)
   if (e == 0) *tcount = 0u;
-  const T* row = nullptr;
+  const double* row = nullptr;
   if constexpr (EB > 0) {
     // rho p of the block's EB elements through shared memory: coalesced loads
     // of the block's contiguous slice of every variable, one row of NP + 1
     // values per element (no bank conflicts when each thread reads its row)
-    __shared__ T s_m[EB > 0 ? EB * (NP + 1) : 1];
+    __shared__ double s_m[EB > 0 ? EB * (NP + 1) : 1];
     const long long e0 = (long long)blockIdx.x * EB;
     const int nel = (int)min((long long)EB, E - e0);
     const size_t vs = (size_t)E * NP;
-    const T gm1 = sizeof(T) == 4 ? T(ma.gamma_f - 1.0f) : T(ma.gamma - 1.0);
+    const double gm1 = ma.gamma - 1.0;
     for (int r = threadIdx.x; r < nel * NP; r += EB) {
       const size_t g = (size_t)e0 * NP + r;
-      T rho, Et, mm = T(0);
-      if constexpr (sizeof(T) == 4) {
-        rho = d2f_int(u[g]);
-        Et = d2f_int(u[(DIM + 1) * vs + g]);
-      } else {
-        rho = u[g];
-        Et = u[(DIM + 1) * vs + g];
-      }
+      const double rho = u[g], Et = u[(DIM + 1) * vs + g];
+      double mm = 0.0;
 #pragma unroll
       for (int k = 0; k < DIM; ++k) {
-        T mk;
-        if constexpr (sizeof(T) == 4) mk = d2f_int(u[(1 + k) * vs + g]);
-        else mk = u[(1 + k) * vs + g];
+        const double mk = u[(1 + k) * vs + g];
         mm += mk * mk;
       }
-      s_m[(r / NP) * (NP + 1) + r % NP] = gm1 * (rho * Et - T(0.5) * mm);
+      s_m[(r / NP) * (NP + 1) + r % NP] = gm1 * (rho * Et - 0.5 * mm);
     }
     __syncthreads();
     row = s_m + threadIdx.x * (NP + 1);
   }
-  auto from_row = [&](int p) { return row[p]; };
   if (e >= E) return;
-  if constexpr (sizeof(R) == 4) {
-    float En;
-    if constexpr (EB > 0) En = indicator_of_values<EQ, N, float>(from_row, lt);
-    else En = indicator_energy<EQ, N, float>(u, E, e, ma, lt);
-    const float a = alpha_of_energy_f32(En, lt);
-    if (a >= 0.0f) {
-      araw[e] = f2d_int(a);
-      return;
-    }
-  }
   double En;
-  if constexpr (sizeof(R) == 8 && EB > 0) En = indicator_of_values<EQ, N, double>(from_row, lt);
-  else En = indicator_energy<EQ, N, double>(u, E, e, ma, lt);
+  if constexpr (EB > 0) En = indicator_of_values<EQ, N, double>([&](int p) { return row[p]; }, lt);
+  else En = indicator_energy<EQ, N>(u, E, e, ma, lt);
   double a = 1.0 / (1.0 + exp(-(lt.sharp / lt.tau) * (En - lt.tau)));
   if (a < 0.001) a = 0.0;
   if (a > 0.999) a = 1.0;

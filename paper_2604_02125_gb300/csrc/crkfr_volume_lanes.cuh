@@ -184,9 +184,9 @@ constexpr int kMinB4 = 3, kMinB4Pack = 2, kMinB5 = 2, kPackMaxN = 4;
 constexpr int kMinB2 = 4, kMinB3 = 3;
 // GLM-MHD (9 variables, 13 pair data): 2 CTAs per SM where the layout allows
 // it, which needs the shared memory of the next tile's staging buffer
-// (128^2, N = 4, FP32: 174 against 206 us per volume launch with one)
+// (128^2, N = 4, FP32: 174 against 206 us per volume launch with one): no such
+// buffer there (PersistLayout::STAGE)
 constexpr int kMinBNc = 2;
-constexpr bool kStageNc = false;
 
 // Kernel shapes: SH = 0 is the measured default of each variant; SH = 1 is the
 // alternative the batched form's autotuner also times: the scalar form (no
@@ -712,7 +712,7 @@ struct PersistLayout {
   using L = LaneLayout<EQ, N, R, SH>;
   static constexpr size_t O_STAGE = (L::bytes() + 15) & ~(size_t)15;
   static constexpr size_t WANT = sizeof(double) * (size_t)EQ::M * L::EPB * L::NP;
-  static constexpr bool STAGE = (!EQ::NC || kStageNc) && O_STAGE + WANT + 16 <= 227 * 1024;
+  static constexpr bool STAGE = !EQ::NC && O_STAGE + WANT + 16 <= 227 * 1024;
   static constexpr size_t STAGE_BYTES = STAGE ? WANT : 0;
   static constexpr size_t O_BAR = O_STAGE + STAGE_BYTES;
   static constexpr size_t bytes() { return O_BAR + 16; }
