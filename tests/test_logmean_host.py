@@ -1,9 +1,12 @@
-"""The FP64 log means' two-part series on the host: the header's own functions,
-compiled as plain C++ with the few device intrinsics they use written out, so
-that their rounding can be compared with exact arithmetic.
+"""The log means' polynomials and the FP64 form's two-part series on the host: the
+coefficients read from the headers against artanh with 40 digits, and the
+header's own functions, compiled as plain C++ with the few device intrinsics
+they use written out, so that their rounding can be compared with exact
+arithmetic.
 """
 import ctypes
 import os
+import re
 import subprocess
 from fractions import Fraction
 
@@ -115,3 +118,37 @@ def test_sums_at_the_ends_of_the_range(host, e):
         e_inv, e_F = _series((Fraction(d[k]) / Fraction(s[k])) ** 2)
         assert abs(4 * Fraction(iF4[k]) - e_inv) <= Fraction(1, 2 ** 52), (e, k, iF4[k])
         assert abs(Fraction(F[k]) - e_F) <= Fraction(1, 2 ** 50), (e, k, F[k])
+
+
+def _coefficients(path, head):
+    """c0, c1, ... of the nested polynomial c0 + u (c1 + u (c2 + ...)) in the function that starts with head,
+    rounded as its suffix says."""
+    with open(path) as f:
+        body = f.read().split(head, 1)[1].split("}", 1)[0]
+    expr = " ".join(re.findall(r"(?:c[0-3]\([^)]*\)|return [^;]*;)", body))
+    vals = []
+    for factor, num, single in re.findall(r"(-?0\.25f \* )?(-?\d+\.\d+)(f?)", expr):
+        v = float(np.float32(num)) if single else float(num)
+        vals.append(float(np.float32(-0.25) * np.float32(v)) if factor else v)
+    return vals if "c3(" not in expr else vals[::-1]
+
+
+@pytest.mark.parametrize("head,umax,kind,bound", [
+    ("double series_F(double u) {", 1 / 16, "F", 1.8e-17), ("double series_invF(double u) {", 1 / 16, "invF", 3.1e-18),
+    ("float series_F(float u) {", 0.05, "F", 1.2e-8), ("float series_invF(float u) {", 0.05, "invF", 3.7e-9),
+    ("float series_invF4(float u) {", 0.05, "invF4", 3.7e-9 / 4),
+    ("f2 series_F(f2 u) {", 0.05, "F", 1.2e-8), ("f2 series_invF4(f2 u) {", 0.05, "invF4", 3.7e-9 / 4)])
+def test_polynomial_errors(head, umax, kind, bound):
+    """The errors stated beside the polynomials, in exact arithmetic."""
+    mp = pytest.importorskip("mpmath")
+    path = HEADER.replace("physics", "f2") if "f2 " in head else HEADER
+    with mp.workdps(40):
+        c = [mp.mpf(x) for x in _coefficients(path, head)]
+        assert len(c) == (9 if umax > 0.06 else 4), c
+        worst = mp.mpf(0)
+        for k in range(1, 801):
+            u = mp.mpf(umax) * (1 - mp.cos(mp.pi * k / 800)) / 2
+            F = mp.atanh(mp.sqrt(u)) / mp.sqrt(u)
+            exact = {"F": F, "invF": 1 / F, "invF4": 1 / (4 * F)}[kind]
+            worst = max(worst, abs(mp.polyval(c[::-1], u) - exact))
+        assert bound / 2 < worst < bound, worst
