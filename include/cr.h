@@ -79,7 +79,8 @@ extern "C" {
 #define CR_LIMITER_BLENDING 1
 
 /* arithmetic of the element-local work */
-#define CR_FP64          0     /* every step of the path in FP64                        */
+#define CR_FP64          0     /* every step of the path to FP64 rounding (terms needed
+                                  to fewer bits may be formed in FP32 parts)            */
 #define CR_FP32_PAIRFLUX 1     /* stages, pair fluxes, time averages and face fluxes in
                                   FP32; the state update u^{n+1} = u^n - dt(...), the dt
                                   reduction and the diagnostic totals stay FP64          */

@@ -421,10 +421,11 @@ struct Euler {
   // stand in for means: f_S,v = f[v] / 2 where half(v), else f[v]; the
   // differentiation coefficients, D_pq and 2 D_pq, carry the factor, so no
   // instruction multiplies by one half.  Kennedy-Gruber: every row halved,
-  // with one addition more -- with two coefficients per pair the front end of
-  // the compiler (CUDA 13.0, its optimisation levels above 1) miscompiled the
-  // branch-free FP32 pair loops of degree 4 and 5 (a constant state lost a
-  // fifth of its mass in a step; the per-variant tests caught it).
+  // with one addition more -- with two coefficients per pair the branch-free FP32
+  // pair loops of degree 4 and 5 gave wrong results at optimisation levels above
+  // 1 (CUDA 13.0; a constant state lost a fifth of its mass in a step, which the
+  // per-variant tests caught).  The cause is not known: the EC flux takes two
+  // coefficients in the same loops and its tests pass.
   __host__ __device__ static constexpr bool half(int v) { return VOL == VOL_KEP || v > 0; }
   template <typename R>
   __device__ __forceinline__ static void two_point(int d, const R* a, const R* b, R* f, const PhysParams<R>& pp) {

@@ -17,7 +17,7 @@
 //    registers; only the y (and z) lines go through shared memory;
 //  * residuals of earlier stages that later stages still need (dense
 //    tableaux, N >= 4) stay with the owner thread;
-//  * 2D Euler in FP32 (N <= 3): the thread's x-line and y-line are
+//  * 2D Euler in FP32 (N <= 4): the thread's x-line and y-line are
 //    flux-differenced together, one in each half of packed FP32x2
 //    instructions (crkfr_f2.cuh), which halves the instructions of the pair
 //    fluxes;
@@ -902,7 +902,8 @@ struct FaceLaneLayout {
 // in whole lines; with a thread per x-line (lane = element) each access of a
 // warp touched 32 different lines, 20 x 32 of them per warp against 72 of the
 // records (2D Euler, N = 3).  us per launch against that form, FP32: 2D Euler
-// 256^2 N = 3 28.4 -> 21.0 (5.8 TB/s of the algorithmic 116 B per node), 128^2 N = 4
+// 256^2 N = 3 28.4 -> 21.0 (launches back to back; 22.4 us after an L2 flush,
+// 5.4 TB/s of the algorithmic 116 B per node), 128^2 N = 4
 // 18.9 -> 12.8, TGV 64^3 649 -> 513, GLM-MHD 128^2 N = 4 57.4 -> 29.0, RKFR 256^2
 // 151 -> 124, 64 batched solves 329 -> 221; FP64 within 4% either way (its
 // FP64 pipe is the bound).
